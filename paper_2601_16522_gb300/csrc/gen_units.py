@@ -12,8 +12,9 @@ device-driven adaptive RKL steps)
 pf_stage_m32k{0,1}   FP32 masked storage, K fixed: fast_kernel<..., true> per
                      pass signature for N <= 4, N <= 32 and N <= 128
 pf_stage_v32k{0,1}   FP32 dense storage, K fixed: vec_kernel (two cells per
-                     thread, N <= 128, nx even) per pass signature followed by
-                     the wide pass of its crowded cells (wide_fix_kernel), and
+                     thread, N <= 128, nx even) per pass signature followed,
+                     where there can be crowded cells, by their wide pass
+                     (wide_fix_kernel), and
                      the _d forms for the device-driven adaptive RKL steps
 """
 import os
@@ -227,7 +228,7 @@ def vunit(kc, fname):
         for sg in FAST_SIGS:
             L.append("    if (g.dim == %d && sig == (%s)) {" % (d, sg))
             L.append("        vec_kernel<%d, %d, %s><<<grid, VBLOCK, vec_smem<%s>(), st>>>(g, P, A, B, L, ptype);" % (d, kc, sg, sg))
-            L.append("        wide_fix_kernel<%d, %d><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);" % (d, kc))
+            L.append("        if (vec_crowds(g)) wide_fix_kernel<%d, %d><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);" % (d, kc))
             L.append("        return (int)cudaGetLastError();")
             L.append("    }")
             prep.append("    if (cudaFuncSetAttribute(vec_kernel<%d, %d, %s>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vec_smem<%s>()) != cudaSuccess) return -1;" % (d, kc, sg, sg))
@@ -253,15 +254,15 @@ def vunit(kc, fname):
     L.append("}")
     L.append("")
     # packed launches of several problems (batched serving)
-    L.append("int launchp_%s(int dim, unsigned sig, const VecInst *tab, const int *bstart, int n, int blocks, int *done," % tag)
-    L.append("             cudaStream_t st, bool *ok)")
+    L.append("int launchp_%s(int dim, unsigned sig, const VecInst *tab, const int *bstart, int n, int blocks, bool crowds," % tag)
+    L.append("             int *done, cudaStream_t st, bool *ok)")
     L.append("{")
     L.append("    *ok = true;")
     for d in (2, 3):
         for sg in FAST_SIGS:
             L.append("    if (dim == %d && sig == (%s)) {" % (d, sg))
             L.append("        packed_kernel<%d, %d, %s><<<blocks, VBLOCK, vec_smem<%s>(), st>>>(tab, bstart, n);" % (d, kc, sg, sg))
-            L.append("        packed_wide_fix_kernel<%d, %d><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);" % (d, kc))
+            L.append("        if (crowds) packed_wide_fix_kernel<%d, %d><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);" % (d, kc))
             L.append("        return (int)cudaGetLastError();")
             L.append("    }")
             prep.append("    if (cudaFuncSetAttribute(packed_kernel<%d, %d, %s>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vec_smem<%s>()) != cudaSuccess) return -1;" % (d, kc, sg, sg))

@@ -27,8 +27,8 @@ int launchd_v32k0(const Geom &, unsigned, const Pass<float> *, cudaStream_t, con
                   const float *, const signed char *, bool *);
 int launchd_v32k1(const Geom &, unsigned, const Pass<float> *, cudaStream_t, const float *, const float *,
                   const float *, const signed char *, bool *);
-int launchp_v32k0(int, unsigned, const VecInst *, const int *, int, int, int *, cudaStream_t, bool *);
-int launchp_v32k1(int, unsigned, const VecInst *, const int *, int, int, int *, cudaStream_t, bool *);
+int launchp_v32k0(int, unsigned, const VecInst *, const int *, int, int, bool, int *, cudaStream_t, bool *);
+int launchp_v32k1(int, unsigned, const VecInst *, const int *, int, int, bool, int *, cudaStream_t, bool *);
 int launch_s32k0(const Geom &, const Pass<float> &, unsigned, cudaStream_t, const float *, const float *,
                  const float *, const signed char *, bool *);
 int launch_s32k1(const Geom &, const Pass<float> &, unsigned, cudaStream_t, const float *, const float *,
@@ -84,7 +84,7 @@ int launch_stage<float>(const Geom &g, const Pass<float> &P, cudaStream_t st, co
         int e = g.K ? launch_v32k1(g, P, sig, st, A, B, L, ptype, &done)
                     : launch_v32k0(g, P, sig, st, A, B, L, ptype, &done);
         if (done) {
-            if (nk) *nk = 2;     // the pass and the wide pass of its crowded cells
+            if (nk) *nk = vec_crowds(g) ? 2 : 1;     // the pass and the wide pass of its crowded cells
             return e;
         }
     }
@@ -117,11 +117,11 @@ int launch_stage_d<float>(const Geom &g, unsigned sig, const Pass<float> *dP, cu
     return g.K ? launchd_f32k1(g, sig, dP, st, A, B, L, ptype) : launchd_f32k0(g, sig, dP, st, A, B, L, ptype);
 }
 
-int launch_packed(int dim, int K, unsigned sig, const VecInst *tab, const int *bstart, int n, int blocks, int *done,
-                  cudaStream_t st, bool *ok)
+int launch_packed(int dim, int K, unsigned sig, const VecInst *tab, const int *bstart, int n, int blocks, bool crowds,
+                  int *done, cudaStream_t st, bool *ok)
 {
-    return K ? launchp_v32k1(dim, sig, tab, bstart, n, blocks, done, st, ok)
-             : launchp_v32k0(dim, sig, tab, bstart, n, blocks, done, st, ok);
+    return K ? launchp_v32k1(dim, sig, tab, bstart, n, blocks, crowds, done, st, ok)
+             : launchp_v32k0(dim, sig, tab, bstart, n, blocks, crowds, done, st, ok);
 }
 
 template <>

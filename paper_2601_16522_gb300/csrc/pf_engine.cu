@@ -656,8 +656,10 @@ int invalidate_mask(pf_handle *h, const void *vecp)
 }
 
 template <typename T>
-int run_pass(pf_handle *h, const Pass<T> &P)
+int run_pass(pf_handle *h, const Pass<T> &P0)
 {
+    Pass<T> P = P0;
+    pfk::finish_pass(P);
     // the kernels evaluate the combination as v + a0 (p0 - v) + a2 (p2 - v)
     if (P.mode == pfk::MODE_STAGE &&
         fabs(P.a1 + (P.p0 ? P.a0 : 0.0) + (P.p2 ? P.a2 : 0.0) - 1.0) > 1e-12)
@@ -1253,6 +1255,7 @@ __global__ void dl_first(DevCtl *c, Pass<T> *d, cudaGraphConditionalHandle hin)
     P.out = (T *)c->buf[w[0]];
     P.r0out = (T *)c->buf[w[3]];
     P.fix_first = o2 ? 1 : 0;
+    pfk::finish_pass(P);
     d[0] = P;
     cudaGraphSetConditional(hin, s >= 2 ? 1u : 0u);
 }
@@ -1292,6 +1295,7 @@ __global__ void dl_stage(DevCtl *c, Pass<T> *d, cudaGraphConditionalHandle hin)
         P.b0 = gt * hs;
     }
     P.out = (T *)c->buf[w[(j - 1) % 3]];
+    pfk::finish_pass(P);
     d[1] = P;
     c->j = j + 1;
     cudaGraphSetConditional(hin, (j + 1 <= s) ? 1u : 0u);
@@ -1314,6 +1318,7 @@ __global__ void dl_err(DevCtl *c, Pass<T> *d)
     P.a_phi = c->tol[1];
     P.r_c = c->tol[2];
     P.a_c = c->tol[3];
+    pfk::finish_pass(P);
     d[2] = P;
 }
 
@@ -2069,6 +2074,7 @@ int pf_create(const pf_params *p, void *cuda_stream, pf_handle **out)
         g.invk[t] = 1.0 / k;
         g.Dk[t] = p->D[t] / k;
     }
+    pfk::finish_geom(g);
     h->dte = gershgorin_dt_e(h, p);
 
     int st = PF_OK;
@@ -2798,7 +2804,7 @@ int batch_round(pf_batch *b)
         !grow(&b->dg, &b->hg, &b->gcap, act.size()) || !grow(&b->dout, &b->hout, &b->ocap, 4 * act.size()))
         return PF_ENOMEM;
     // waves: the w-th pass of every request; one packed launch per pass kind
-    struct Launch { int dim, K; unsigned sig; size_t toff; int n, blocks; };
+    struct Launch { int dim, K; unsigned sig; size_t toff; int n, blocks; bool crowds; };
     std::vector<Launch> launches;
     size_t toff = 0;
     for (size_t w = 0; w < maxw; ++w) {
@@ -2809,7 +2815,7 @@ int batch_round(pf_batch *b)
                 groups[std::make_tuple(r.h->g.dim, r.h->K, pfk::pass_signature(r.passes[w]))].push_back(k);
         }
         for (auto &gr : groups) {
-            Launch l{std::get<0>(gr.first), std::get<1>(gr.first), std::get<2>(gr.first), toff, 0, 0};
+            Launch l{std::get<0>(gr.first), std::get<1>(gr.first), std::get<2>(gr.first), toff, 0, 0, false};
             for (int k : gr.second) {
                 BatchReq &r = b->slots[k];
                 pfk::VecInst &I = b->htab[toff];
@@ -2824,7 +2830,9 @@ int batch_round(pf_batch *b)
                 l.blocks += I.nblk;
                 l.n++;
                 toff++;
-                r.launches += 2;
+                const bool crowds = pfk::vec_crowds(r.h->g);
+                l.crowds = l.crowds || crowds;
+                r.launches += crowds ? 2 : 1;
             }
             launches.push_back(l);
         }
@@ -2836,7 +2844,7 @@ int batch_round(pf_batch *b)
     for (const Launch &l : launches) {
         bool ok = false;
         const int e = pfk::launch_packed(l.dim, l.K, l.sig, b->dtab + l.toff, b->dstart + l.toff, l.n, l.blocks,
-                                         b->ddone, b->stream, &ok);
+                                         l.crowds, b->ddone, b->stream, &ok);
         if (!ok || e != 0) return PF_EDEVICE;
     }
     // error partials and status words of every request, one transfer

@@ -32,11 +32,12 @@ int launch_stage_d(const Geom &g, unsigned sig, const Pass<T> *dP, cudaStream_t 
 
 // Packed launch of one pass kind (dimension dim, K, signature sig) over the n
 // problems of a device table (two-cell FP32 passes; see VecInst): blocks is
-// the sum of their block counts, bstart their prefix sums, done a zeroed
-// device counter of the caller.  Returns a cudaError_t; *ok false when the
+// the sum of their block counts, bstart their prefix sums, crowds whether any
+// of them can have crowded cells (vec_crowds), done a zeroed device counter of
+// the caller.  Returns a cudaError_t; *ok false when the
 // pass kind has no packed form.
-int launch_packed(int dim, int K, unsigned sig, const VecInst *tab, const int *bstart, int n, int blocks, int *done,
-                  cudaStream_t st, bool *ok);
+int launch_packed(int dim, int K, unsigned sig, const VecInst *tab, const int *bstart, int n, int blocks, bool crowds,
+                  int *done, cudaStream_t st, bool *ok);
 
 // Opt every instantiation into its shared memory on the current device;
 // returns the resident blocks per SM of the generic 3D kernel (<= 0: error).

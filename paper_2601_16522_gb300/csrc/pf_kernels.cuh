@@ -49,18 +49,27 @@ __device__ __forceinline__ T affine(T v, T p0, T p2, T a0, T a2)
     return acc;
 }
 
+// Problem constants in the arithmetic type of a pass, converted once on the
+// host.  GB300 issues an FP64 warp instruction (conversions included) about
+// once in 16 cycles per SM, so an FP32 pass that converted or divided FP64
+// constants per thread spent most of its time on them (RKL2 pass at 256^3 x
+// 32, FP32: 2.27 ms with the conversions in the kernel).
+template <typename T>
+struct GeomConst {
+    T dx2, idx2;                        // dx * dx and 1 / dx^2 (rounded from FP64)
+    T k[2], c0[2], invk[2], Dk[2];      // per chemical type: k, c0 - cref, 1/k, D/k
+    T cdir[6];                          // Dirichlet value of c per face, minus cref
+    T cref;                             // FP32 storage holds c - cref (0 in FP64); c0 and cdir
+                                        // are shifted by it, so mu and the face fluxes are those
+                                        // of c, and only the error weights |c| add it back
+};
+
 // Problem constants shared by every pass (passed by value).
-struct Geom {
+struct Geom : GeomConst<double> {
     int nx, ny, nz, dim;
     long long V, Vs;                    // cells, field stride
     int N, K, NF;
     int bc_phi[6], bc_c[6];
-    double cdir[6];                     // Dirichlet value of c per face, minus cref
-    double dx2;                         // dx * dx
-    double k[2], c0[2], invk[2], Dk[2]; // per chemical type: k, c0 - cref, 1/k, D/k
-    double cref;                        // FP32 storage holds c - cref (0 in FP64); c0 and cdir
-                                        // are shifted by it, so mu and the face fluxes are those
-                                        // of c, and only the error weights |c| add it back
     int tiles_x, tiles_y;               // block tiling of the x-y plane (one-cell kernels)
     int kvar;                           // FP32 dense passes: KVAR_TWO_CELL or KVAR_ONE_CELL
     int simplex;                        // projection S: SIMPLEX_STANDARD or SIMPLEX_MOBILITY
@@ -68,13 +77,45 @@ struct Geom {
     int uni;                            // slot passes: 1 if every off-diagonal entry of each
     float uA, uB, uL;                   // FP32 table A, B, L is the same value (these), which
                                         // the pairwise sums then use instead of gathers
+    GeomConst<float> cf;                // the FP64 constants of the base, as float
 };
+
+template <typename T> __device__ __forceinline__ const GeomConst<T> &geom_const(const Geom &g);
+template <> __device__ __forceinline__ const GeomConst<float> &geom_const<float>(const Geom &g) { return g.cf; }
+template <> __device__ __forceinline__ const GeomConst<double> &geom_const<double>(const Geom &g) { return g; }
+
+// Completes the derived constants once the FP64 ones are set.
+inline void finish_geom(Geom &g)
+{
+    g.idx2 = 1.0 / g.dx2;
+    GeomConst<float> &c = g.cf;
+    c.idx2 = (float)g.idx2;
+    c.dx2 = (float)g.dx2;
+    for (int t = 0; t < 2; ++t) {
+        c.k[t] = (float)g.k[t];
+        c.c0[t] = (float)g.c0[t];
+        c.invk[t] = (float)g.invk[t];
+        c.Dk[t] = (float)g.Dk[t];
+    }
+    for (int f = 0; f < 6; ++f) c.cdir[f] = (float)g.cdir[f];
+    c.cref = (float)g.cref;
+}
+
 // Kernel variants of the FP32 dense passes (chosen per handle, pf_autotune).
 enum { KVAR_TWO_CELL = 0, KVAR_ONE_CELL = 1 };
 // The projection onto the simplex after every stage (Sec. 3.1): the standard
 // one (clamp, >= 1 rule, divide by the sum) or the mobility-weighted one
 // (mob_project; the generic body only).
 enum { SIMPLEX_STANDARD = 0, SIMPLEX_MOBILITY = 1 };
+
+// Scalars of one pass in its arithmetic type (see GeomConst); written from
+// the FP64 values by finish_pass, on the host or by a planning kernel.
+template <typename T>
+struct PassConst {
+    T a0, a2, b1, b0, bz, m25, m15;
+    T ib1;                              // 1 / b1, divided in FP64 (first-stage fix)
+    T dt, r_phi, a_phi, r_c, a_c;
+};
 
 // What one pass does (passed by value).
 template <typename T>
@@ -116,7 +157,18 @@ struct Pass {
     // the same for the SSP(10)4 vectors: z accumulator in/out, q2 in/out, u^n
     const unsigned *m_zin, *m_q2in, *m_uw;
     unsigned *m_zout, *m_out2;
+    PassConst<T> c;      // the scalars above as T (finish_pass)
 };
+
+template <typename T>
+__host__ __device__ inline void finish_pass(Pass<T> &P)
+{
+    P.c.a0 = (T)P.a0; P.c.a2 = (T)P.a2; P.c.b1 = (T)P.b1; P.c.b0 = (T)P.b0; P.c.bz = (T)P.bz;
+    P.c.m25 = (T)P.m25; P.c.m15 = (T)P.m15;
+    P.c.ib1 = (T)(1.0 / P.b1);
+    P.c.dt = (T)P.dt;
+    P.c.r_phi = (T)P.r_phi; P.c.a_phi = (T)P.a_phi; P.c.r_c = (T)P.r_c; P.c.a_c = (T)P.a_c;
+}
 
 enum { MODE_RHS = 0, MODE_STAGE = 1, MODE_ERR = 2 };
 
@@ -142,15 +194,16 @@ __device__ __forceinline__ void raise_flag(int *flag, int bits)
 }
 
 // End of a pass that completes a fixed step (every thread of the block calls
-// it): the last block of the grid to finish counts the step.  A flag raised
+// it): the last block of the pass (of nblk; -1: the whole grid) to finish
+// counts the step.  A flag raised
 // during the pass is recorded (raise_flag) before the raising block finishes,
 // hence before the count moves on.
-__device__ __forceinline__ void count_step_done(int *flag)
+__device__ __forceinline__ void count_step_done(int *flag, int nblk = -1)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
+        const unsigned nb = nblk >= 0 ? (unsigned)nblk : gridDim.x * gridDim.y * gridDim.z;
         if (atomicAdd((unsigned *)(flag + 2), 1u) == nb - 1u) {
             atomicExch(flag + 2, 0);
             atomicAdd(flag + 1, 1);
@@ -456,7 +509,8 @@ __device__ __forceinline__ bool cell_core(const Geom &g, const Pass<T> &P, LST &
     const int K = KC;
     const long long Vs = g.Vs;
     const long long i = ((long long)z * g.ny + y) * g.nx + x;
-    const T dx2 = (T)g.dx2;
+    const GeomConst<T> &gc = geom_const<T>(g);
+    const T dx2 = gc.dx2;
 
     long long off[6];
     int ghost[6];
@@ -476,7 +530,7 @@ __device__ __forceinline__ bool cell_core(const Geom &g, const Pass<T> &P, LST &
 #pragma unroll
         for (int f = 0; f < NFACE; ++f) {
             T v = ldg(cf + off[f]);
-            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * (T)g.cdir[f] - cc;
+            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * gc.cdir[f] - cc;
             num_n[f] = v;
         }
     }
@@ -494,7 +548,7 @@ __device__ __forceinline__ bool cell_core(const Geom &g, const Pass<T> &P, LST &
             const bool act = nontrivial<NFACE>(v0, nb);
             if (K) {
                 const int t = ptype[a];
-                const T c0t = (T)g.c0[t], ikt = (T)g.invk[t], dkt = (T)g.Dk[t];
+                const T c0t = gc.c0[t], ikt = gc.invk[t], dkt = gc.Dk[t];
                 num_c = num_c - v0 * c0t;
                 den_c = den_c + v0 * ikt;
 #pragma unroll
@@ -545,7 +599,7 @@ __device__ __forceinline__ bool cell_core(const Geom &g, const Pass<T> &P, LST &
         T psi = (T)0;
         if (K) {
             const int t = ptype[a];
-            psi = -(mu * mu) / ((T)2 * (T)g.k[t]) - mu * (T)g.c0[t];
+            psi = -(mu * mu) / ((T)2 * gc.k[t]) - mu * gc.c0[t];
         }
         S.dl(k) = d + psi;
     }
@@ -588,8 +642,8 @@ __device__ __forceinline__ bool cell_core(const Geom &g, const Pass<T> &P, LST &
         if (P.nz_out) P.nz_out[i] = (unsigned char)nz;
     } else if (mode == MODE_ERR) {
         // ---- STS error sweep (Sec. 3.3): in = u^{n+1}, p0 = u^n, r0in = F^n
-        const T dt = (T)P.dt;
-        const T rph = (T)P.r_phi, aph = (T)P.a_phi;
+        const T dt = P.c.dt;
+        const T rph = P.c.r_phi, aph = P.c.a_phi;
         int nc = 0;
         long long o = i;
 #pragma unroll 4
@@ -619,15 +673,15 @@ __device__ __forceinline__ bool cell_core(const Geom &g, const Pass<T> &P, LST &
             const T un = ldg(P.p0 + oc), un1 = ldg(P.in + oc), rn = ldg(P.r0in + oc);
             const T sr = rn + rc;
             const T e = ((T)12 * (un - un1) + ((T)6 * dt) * sr) / (T)15;
-            const T au = tabs(un + (T)g.cref), av = tabs(un1 + (T)g.cref);
-            const T w = (T)P.r_c * (au > av ? au : av) + (T)P.a_c;
+            const T au = tabs(un + gc.cref), av = tabs(un1 + gc.cref);
+            const T w = P.c.r_c * (au > av ? au : av) + P.c.a_c;
             const T q = e / w;
             esum += (double)(q * q);
             ecnt += 1;
         }
     } else {
         // ---- stage combination (Eq. sts / Alg. ssp2 / SSP(10)4) -------------
-        const T a0c = (T)P.a0, a2c = (T)P.a2, b1c = (T)P.b1, b0c = (T)P.b0, bzc = (T)P.bz;
+        const T a0c = P.c.a0, a2c = P.c.a2, b1c = P.c.b1, b0c = P.c.b0, bzc = P.c.bz;
         // the mobility-weighted projection works on the stage values in the output
         const bool mob = GEN && project && g.simplex == SIMPLEX_MOBILITY;
         const bool chunked = N > NV || mob;
@@ -711,16 +765,16 @@ __device__ __forceinline__ bool cell_core(const Geom &g, const Pass<T> &P, LST &
                     if (zv < (T)0 || zv > (T)1) e = (T)0;
                     if (e != (T)0) {
                         const T au = tabs(ldg(P.uw + o)), av = tabs(w);
-                        const T wt = (T)P.r_phi * (au > av ? au : av) + (T)P.a_phi;
+                        const T wt = P.c.r_phi * (au > av ? au : av) + P.c.a_phi;
                         const T q = e / wt;
                         esum += (double)(q * q);
                         nc++;
                     }
                 }
                 if (has_out2) {
-                    const T q2 = w + (T)P.m25 * (ldg(P.q2in + o) - w);
+                    const T q2 = w + P.c.m25 * (ldg(P.q2in + o) - w);
                     P.out2[o] = q2;
-                    P.out[o] = w + (T)P.m15 * (q2 - w);
+                    P.out[o] = w + P.c.m15 * (q2 - w);
                 } else {
                     P.out[o] = w;
                 }
@@ -743,17 +797,17 @@ __device__ __forceinline__ bool cell_core(const Geom &g, const Pass<T> &P, LST &
                 P.zout[o] = zv;
                 if (emb) {
                     const T e = acc - zv;
-                    const T au = tabs(ldg(P.uw + o) + (T)g.cref), av = tabs(acc + (T)g.cref);
-                    const T wt = (T)P.r_c * (au > av ? au : av) + (T)P.a_c;
+                    const T au = tabs(ldg(P.uw + o) + gc.cref), av = tabs(acc + gc.cref);
+                    const T wt = P.c.r_c * (au > av ? au : av) + P.c.a_c;
                     const T q = e / wt;
                     esum += (double)(q * q);
                     ecnt += 1;
                 }
             }
             if (has_out2) {
-                const T q2 = acc + (T)P.m25 * (ldg(P.q2in + o) - acc);
+                const T q2 = acc + P.c.m25 * (ldg(P.q2in + o) - acc);
                 P.out2[o] = q2;
-                P.out[o] = acc + (T)P.m15 * (q2 - acc);
+                P.out[o] = acc + P.c.m15 * (q2 - acc);
             } else {
                 P.out[o] = acc;
             }
@@ -1045,10 +1099,11 @@ __device__ __forceinline__ bool fast_cell(const Geom &g, const Pass<float> &P, L
     const int N = g.N;
     const int Vs = (int)g.Vs;
     const int i32 = (int)i;
-    const T idx2 = (T)(1.0 / g.dx2);
-    const T a0c = (T)P.a0, a2c = (T)P.a2, b1c = (T)P.b1, b0c = (T)P.b0;
-    const T ib1 = (T)(1.0 / P.b1);   // first-stage fix: F <- (S(u1) - u^n) / (mu~_1 dt)
-    const T dt = (T)P.dt, rph = (T)P.r_phi, aph = (T)P.a_phi;
+    const GeomConst<T> &gc = geom_const<T>(g);
+    const T idx2 = gc.idx2;
+    const T a0c = P.c.a0, a2c = P.c.a2, b1c = P.c.b1, b0c = P.c.b0;
+    const T ib1 = P.c.ib1;   // first-stage fix: F <- (S(u1) - u^n) / (mu~_1 dt)
+    const T dt = P.c.dt, rph = P.c.r_phi, aph = P.c.a_phi;
 
     // concentration
     T cc = (T)0, num_c = (T)0, den_c = (T)0, num_n[NFACE], den_n[NFACE], mf[NFACE];
@@ -1061,7 +1116,7 @@ __device__ __forceinline__ bool fast_cell(const Geom &g, const Pass<float> &P, L
 #pragma unroll
         for (int f = 0; f < NFACE; ++f) {
             T v = ldg(cf + off[f]);
-            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * (T)g.cdir[f] - cc;
+            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * gc.cdir[f] - cc;
             num_n[f] = v;
         }
     }
@@ -1088,7 +1143,7 @@ __device__ __forceinline__ bool fast_cell(const Geom &g, const Pass<float> &P, L
             }
             if (KC) {
                 const int t = ptype[a];
-                const T c0t = (T)g.c0[t], ikt = (T)g.invk[t], dkt = (T)g.Dk[t];
+                const T c0t = gc.c0[t], ikt = gc.invk[t], dkt = gc.Dk[t];
                 num_c = num_c - v0 * c0t;
                 den_c = den_c + v0 * ikt;
 #pragma unroll
@@ -1158,7 +1213,7 @@ __device__ __forceinline__ bool fast_cell(const Geom &g, const Pass<float> &P, L
         }
         if (KC) {
             const int t = ptype[a];
-            d = d + (-(mu * mu) / ((T)2 * (T)g.k[t]) - mu * (T)g.c0[t]);
+            d = d + (-(mu * mu) / ((T)2 * gc.k[t]) - mu * gc.c0[t]);
         }
         S.dl[k][tid] = d;
     }
@@ -1199,7 +1254,7 @@ __device__ __forceinline__ bool fast_cell(const Geom &g, const Pass<float> &P, L
             const long long o = (long long)N * Vs + i;
             const T un = ldg(P.p0 + o), un1 = cc, rn = ldg(P.r0in + o);
             const T e = ((T)12 * (un - un1) + ((T)6 * dt) * (rn + rc)) * ((T)1 / (T)15);
-            const T w = (T)P.r_c * fmaxf(fabsf(un + (T)g.cref), fabsf(un1 + (T)g.cref)) + (T)P.a_c;
+            const T w = P.c.r_c * fmaxf(fabsf(un + gc.cref), fabsf(un1 + gc.cref)) + P.c.a_c;
             const T q = e / w;
             esum += (double)(q * q);
             ecnt += 1;
@@ -1305,11 +1360,12 @@ __device__ __forceinline__ void masked_cell(const Geom &g, const Pass<float> &P,
     const int N = g.N;
     const int Vs = (int)g.Vs;
     const int i32 = (int)i;
-    const T idx2 = (T)(1.0 / g.dx2);
-    const T a0c = (T)P.a0, a2c = (T)P.a2, b1c = (T)P.b1, b0c = (T)P.b0;
-    const T ib1 = (T)(1.0 / P.b1);   // first-stage fix: F <- (S(u1) - u^n) / (mu~_1 dt)
-    const T dt = (T)P.dt, rph = (T)P.r_phi, aph = (T)P.a_phi;
-    const T bzc = (T)P.bz, m25 = (T)P.m25, m15 = (T)P.m15;
+    const GeomConst<T> &gc = geom_const<T>(g);
+    const T idx2 = gc.idx2;
+    const T a0c = P.c.a0, a2c = P.c.a2, b1c = P.c.b1, b0c = P.c.b0;
+    const T ib1 = P.c.ib1;   // first-stage fix: F <- (S(u1) - u^n) / (mu~_1 dt)
+    const T dt = P.c.dt, rph = P.c.r_phi, aph = P.c.a_phi;
+    const T bzc = P.c.bz, m25 = P.c.m25, m15 = P.c.m15;
 
     // concentration
     T cc = (T)0, num_c = (T)0, den_c = (T)0, num_n[NFACE], den_n[NFACE], mf[NFACE];
@@ -1322,7 +1378,7 @@ __device__ __forceinline__ void masked_cell(const Geom &g, const Pass<float> &P,
 #pragma unroll
         for (int f = 0; f < NFACE; ++f) {
             T v = ldg(cf + off[f]);
-            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * (T)g.cdir[f] - cc;
+            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * gc.cdir[f] - cc;
             num_n[f] = v;
         }
     }
@@ -1397,7 +1453,7 @@ __device__ __forceinline__ void masked_cell(const Geom &g, const Pass<float> &P,
         }
         if (KC) {
             const int t = ptype[a];
-            const T c0t = (T)g.c0[t], ikt = (T)g.invk[t], dkt = (T)g.Dk[t];
+            const T c0t = gc.c0[t], ikt = gc.invk[t], dkt = gc.Dk[t];
             num_c = num_c - v0 * c0t;
             den_c = den_c + v0 * ikt;
 #pragma unroll
@@ -1471,7 +1527,7 @@ __device__ __forceinline__ void masked_cell(const Geom &g, const Pass<float> &P,
         }
         if (KC) {
             const int t = ptype[a];
-            d = d + (-(mu * mu) / ((T)2 * (T)g.k[t]) - mu * (T)g.c0[t]);
+            d = d + (-(mu * mu) / ((T)2 * gc.k[t]) - mu * gc.c0[t]);
         }
         S.dl[k][tid] = d;
     }
@@ -1523,7 +1579,7 @@ __device__ __forceinline__ void masked_cell(const Geom &g, const Pass<float> &P,
             const long long o = (long long)N * Vs + i;
             const T un = ldg(P.p0 + o), un1 = cc, rn = ldg(P.r0in + o);
             const T e = ((T)12 * (un - un1) + ((T)6 * dt) * (rn + rc)) * ((T)1 / (T)15);
-            const T wt = (T)P.r_c * fmaxf(fabsf(un + (T)g.cref), fabsf(un1 + (T)g.cref)) + (T)P.a_c;
+            const T wt = P.c.r_c * fmaxf(fabsf(un + gc.cref), fabsf(un1 + gc.cref)) + P.c.a_c;
             const T q = e / wt;
             esum += (double)(q * q);
             ecnt += 1;
@@ -1654,8 +1710,8 @@ __device__ __forceinline__ void masked_cell(const Geom &g, const Pass<float> &P,
             if (!over) P.zout[o] = zv;
             if (EMB) {
                 const T e = acc - zv;
-                const T au = fabsf(ldg(P.uw + o) + (T)g.cref), av = fabsf(acc + (T)g.cref);
-                const T wt = (T)P.r_c * fmaxf(au, av) + (T)P.a_c;
+                const T au = fabsf(ldg(P.uw + o) + gc.cref), av = fabsf(acc + gc.cref);
+                const T wt = P.c.r_c * fmaxf(au, av) + P.c.a_c;
                 const T q = e / wt;
                 esum += (double)(q * q);
                 ecnt += 1;
@@ -1694,10 +1750,11 @@ __device__ __forceinline__ bool big_cell(const Geom &g, const Pass<float> &P, Pl
     const int N = g.N;
     const long long Vs = g.Vs;
     const int i32 = (int)i;
-    const T idx2 = (T)(1.0 / g.dx2);
-    const T a0c = (T)P.a0, a2c = (T)P.a2, b1c = (T)P.b1, b0c = (T)P.b0;
-    const T ib1 = (T)(1.0 / P.b1);   // first-stage fix: F <- (S(u1) - u^n) / (mu~_1 dt)
-    const T dt = (T)P.dt, rph = (T)P.r_phi, aph = (T)P.a_phi;
+    const GeomConst<T> &gc = geom_const<T>(g);
+    const T idx2 = gc.idx2;
+    const T a0c = P.c.a0, a2c = P.c.a2, b1c = P.c.b1, b0c = P.c.b0;
+    const T ib1 = P.c.ib1;   // first-stage fix: F <- (S(u1) - u^n) / (mu~_1 dt)
+    const T dt = P.c.dt, rph = P.c.r_phi, aph = P.c.a_phi;
     auto combo = [&](T p0v, T v0, T p2v, T r0v) {
         T acc = affine<HP0, HP2>(v0, p0v, p2v, a0c, a2c);
         if (HR0) acc = acc + b0c * r0v;
@@ -1714,7 +1771,7 @@ __device__ __forceinline__ bool big_cell(const Geom &g, const Pass<float> &P, Pl
 #pragma unroll
         for (int f = 0; f < NFACE; ++f) {
             T v = ldg(cf + off[f]);
-            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * (T)g.cdir[f] - cc;
+            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * gc.cdir[f] - cc;
             num_n[f] = v;
         }
     }
@@ -1739,7 +1796,7 @@ __device__ __forceinline__ bool big_cell(const Geom &g, const Pass<float> &P, Pl
                 }
                 if (KC) {
                     const int t = ptype[a];
-                    const T c0t = (T)g.c0[t], ikt = (T)g.invk[t], dkt = (T)g.Dk[t];
+                    const T c0t = gc.c0[t], ikt = gc.invk[t], dkt = gc.Dk[t];
                     num_c = num_c - v0 * c0t;
                     den_c = den_c + v0 * ikt;
 #pragma unroll
@@ -1803,7 +1860,7 @@ __device__ __forceinline__ bool big_cell(const Geom &g, const Pass<float> &P, Pl
         }
         if (KC) {
             const int t = ptype[a];
-            d = d + (-(mu * mu) / ((T)2 * (T)g.k[t]) - mu * (T)g.c0[t]);
+            d = d + (-(mu * mu) / ((T)2 * gc.k[t]) - mu * gc.c0[t]);
         }
         S.dl[k][tid] = d;
     }
@@ -1851,7 +1908,7 @@ __device__ __forceinline__ bool big_cell(const Geom &g, const Pass<float> &P, Pl
             const long long o = (long long)N * Vs + i;
             const T un = ldg(P.p0 + o), un1 = cc, rn = ldg(P.r0in + o);
             const T e = ((T)12 * (un - un1) + ((T)6 * dt) * (rn + rc)) * ((T)1 / (T)15);
-            const T w = (T)P.r_c * fmaxf(fabsf(un + (T)g.cref), fabsf(un1 + (T)g.cref)) + (T)P.a_c;
+            const T w = P.c.r_c * fmaxf(fabsf(un + gc.cref), fabsf(un1 + gc.cref)) + P.c.a_c;
             const T q = e / w;
             esum += (double)(q * q);
             ecnt += 1;

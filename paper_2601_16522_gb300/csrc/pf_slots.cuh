@@ -124,10 +124,11 @@ __device__ __forceinline__ bool slot_cell(const Geom &g, const Pass<float> &P, L
     const int N = g.N;
     const int Vs = (int)g.Vs;
     const long long co = (long long)SLOT_C_PLANES * Vs;   // concentration plane
-    const T idx2 = (T)(1.0 / g.dx2);
-    const T a0c = (T)P.a0, a2c = (T)P.a2, b1c = (T)P.b1, b0c = (T)P.b0;
-    const T ib1 = (T)(1.0 / P.b1);   // first-stage fix: F <- (S(u1) - u^n) / (mu~_1 dt)
-    const T dt = (T)P.dt, rph = (T)P.r_phi, aph = (T)P.a_phi;
+    const GeomConst<T> &gc = geom_const<T>(g);
+    const T idx2 = gc.idx2;
+    const T a0c = P.c.a0, a2c = P.c.a2, b1c = P.c.b1, b0c = P.c.b0;
+    const T ib1 = P.c.ib1;   // first-stage fix: F <- (S(u1) - u^n) / (mu~_1 dt)
+    const T dt = P.c.dt, rph = P.c.r_phi, aph = P.c.a_phi;
 
     // concentration
     T cc = (T)0, num_c = (T)0, den_c = (T)0, num_n[NFACE], den_n[NFACE], mf[NFACE];
@@ -140,7 +141,7 @@ __device__ __forceinline__ bool slot_cell(const Geom &g, const Pass<float> &P, L
 #pragma unroll
         for (int f = 0; f < NFACE; ++f) {
             T v = ldg(cf + off[f]);
-            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * (T)g.cdir[f] - cc;
+            if (ghost[f] && g.bc_c[f] == BC_DIRICHLET) v = (T)2 * gc.cdir[f] - cc;
             num_n[f] = v;
         }
     }
@@ -192,7 +193,7 @@ __device__ __forceinline__ bool slot_cell(const Geom &g, const Pass<float> &P, L
         }
         if (KC) {
             const int t = ptype[a];
-            const T c0t = (T)g.c0[t], ikt = (T)g.invk[t], dkt = (T)g.Dk[t];
+            const T c0t = gc.c0[t], ikt = gc.invk[t], dkt = gc.Dk[t];
             num_c = num_c - v0 * c0t;
             den_c = den_c + v0 * ikt;
 #pragma unroll
@@ -267,7 +268,7 @@ __device__ __forceinline__ bool slot_cell(const Geom &g, const Pass<float> &P, L
         }
         if (KC) {
             const int t = ptype[a];
-            d = d + (-(mu * mu) / ((T)2 * (T)g.k[t]) - mu * (T)g.c0[t]);
+            d = d + (-(mu * mu) / ((T)2 * gc.k[t]) - mu * gc.c0[t]);
         }
         S.dl(k) = d;
     }
@@ -313,7 +314,7 @@ __device__ __forceinline__ bool slot_cell(const Geom &g, const Pass<float> &P, L
         if (KC) {
             const T un = ldg(P.p0 + co + i), un1 = cc, rn = ldg(P.r0in + co + i);
             const T e = ((T)12 * (un - un1) + ((T)6 * dt) * (rn + rc)) * ((T)1 / (T)15);
-            const T wt = (T)P.r_c * fmaxf(fabsf(un + (T)g.cref), fabsf(un1 + (T)g.cref)) + (T)P.a_c;
+            const T wt = P.c.r_c * fmaxf(fabsf(un + gc.cref), fabsf(un1 + gc.cref)) + P.c.a_c;
             const T q = e / wt;
             esum += (double)(q * q);
             ecnt += 1;

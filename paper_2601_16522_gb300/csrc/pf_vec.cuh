@@ -78,6 +78,13 @@ __host__ __device__ inline bool vec_eligible(const Geom &g)
     return (g.nx % 2) == 0 && g.N <= 128 && g.V < 0x7fffffffLL;
 }
 
+// Problems of at most this many phases have no crowded cells (every list
+// holds them all): their passes need no wide pass after them, which at small
+// grids is half of the launches (2D circle 128^2, RKL2: 5.8 us for a pass,
+// 2.5 us and a launch for the wide pass that finds nothing).
+constexpr int VEC_NO_CROWD = PF_VEC_ACT < PF_VEC_ACT_LIGHT ? PF_VEC_ACT : PF_VEC_ACT_LIGHT;
+__host__ __device__ inline bool vec_crowds(const Geom &g) { return g.N > VEC_NO_CROWD; }
+
 // Whether a pass is one of the heavy ones (two extra pointwise streams).
 template <unsigned SIG>
 __host__ __device__ constexpr bool vec_heavy() { return (SIG & (SIG_P0 | SIG_P2)) == (SIG_P0 | SIG_P2); }
@@ -194,10 +201,11 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
         const bool lneed = here && !lsh && !lself, rneed = here && !rsh && !rself;
         const int lofs = x > 0 ? -1 : g.nx - 1;
         const int rofs = x + 2 < g.nx ? 2 : 2 - g.nx;
-        const T idx2 = (T)(1.0 / g.dx2);
-        const T a0c = (T)P.a0, a2c = (T)P.a2, b1c = (T)P.b1, b0c = (T)P.b0;
-        const T ib1 = (T)(1.0 / P.b1);
-        const T dt = (T)P.dt, rph = (T)P.r_phi, aph = (T)P.a_phi;
+        const GeomConst<T> &gc = geom_const<T>(g);
+        const T idx2 = gc.idx2;
+        const T a0c = P.c.a0, a2c = P.c.a2, b1c = P.c.b1, b0c = P.c.b0;
+        const T ib1 = P.c.ib1;
+        const T dt = P.c.dt, rph = P.c.r_phi, aph = P.c.a_phi;
 
         // concentration: per chemical type, phase sums of the two cells, of
         // their y/z neighbours and of the x edge cells
@@ -355,8 +363,8 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
         // ---- concentration: mu of the cells and their neighbours, c RHS ------
         T mu[2] = {(T)0, (T)0}, rc[2] = {(T)0, (T)0}, cc[2] = {(T)0, (T)0};
         if (KC) {
-            const T c00 = (T)g.c0[0], c01 = (T)g.c0[1], ik0 = (T)g.invk[0], ik1 = (T)g.invk[1];
-            const T dk0 = (T)g.Dk[0], dk1 = (T)g.Dk[1];
+            const T c00 = gc.c0[0], c01 = gc.c0[1], ik0 = gc.invk[0], ik1 = gc.invk[1];
+            const T dk0 = gc.Dk[0], dk1 = gc.Dk[1];
             const float *cf = P.in + (long long)N * Vs + i;
             float2 c2 = make_float2(0.f, 0.f), cym = c2, cyp = c2, czm = c2, czp = c2;
             float cel = 0.f, cer = 0.f;
@@ -388,12 +396,12 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
             if (lsh) { mul = mul_s; Ml = Ml_s; }
             else if (lself) {
                 // zero-gradient phi; c Dirichlet (ghost 2 c_b - c) or zero-gradient
-                mul = g.bc_c[0] == BC_DIRICHLET ? muof((T)2 * (T)g.cdir[0] - cc[0], Ph[0]) : mu[0];
+                mul = g.bc_c[0] == BC_DIRICHLET ? muof((T)2 * gc.cdir[0] - cc[0], Ph[0]) : mu[0];
                 Ml = M[0];
             } else { mul = muof(cel, Pe[0]); Ml = mof(Pe[0]); }
             if (rsh) { mur = mur_s; Mr = Mr_s; }
             else if (rself) {
-                mur = g.bc_c[1] == BC_DIRICHLET ? muof((T)2 * (T)g.cdir[1] - cc[1], Ph[1]) : mu[1];
+                mur = g.bc_c[1] == BC_DIRICHLET ? muof((T)2 * gc.cdir[1] - cc[1], Ph[1]) : mu[1];
                 Mr = M[1];
             } else { mur = muof(cer, Pe[1]); Mr = mof(Pe[1]); }
             const float2 cnb[4] = {cym, cyp, czm, czp};
@@ -409,7 +417,7 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
 #pragma unroll
                 for (int f = 0; f < 2 * (DIM - 1); ++f) {
                     T cv = c == 0 ? cnb[f].x : cnb[f].y;
-                    if (ghost[2 + f] && g.bc_c[2 + f] == BC_DIRICHLET) cv = (T)2 * (T)g.cdir[2 + f] - cc[c];
+                    if (ghost[2 + f] && g.bc_c[2 + f] == BC_DIRICHLET) cv = (T)2 * gc.cdir[2 + f] - cc[c];
                     const T mun = muof(cv, Pn[c][f]);
                     acc = acc + ((T)0.5 * (M[c] + mof(Pn[c][f]))) * (mun - mu[c]);
                 }
@@ -436,7 +444,7 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                 }
                 if (KC) {
                     const int t = ptype[a];
-                    d = d + (-(mu[c] * mu[c]) / ((T)2 * (T)g.k[t]) - mu[c] * (T)g.c0[t]);
+                    d = d + (-(mu[c] * mu[c]) / ((T)2 * gc.k[t]) - mu[c] * gc.c0[t]);
                 }
                 S.dl[k][slot] = d;
             }
@@ -497,7 +505,7 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                     const long long o = (long long)N * Vs + i + c;
                     const T un = __ldg(P.p0 + o), un1 = cc[c], rn = __ldg(P.r0in + o);
                     const T e = ((T)12 * (un - un1) + ((T)6 * dt) * (rn + rc[c])) * ((T)1 / (T)15);
-                    const T w = (T)P.r_c * fmaxf(fabsf(un + (T)g.cref), fabsf(un1 + (T)g.cref)) + (T)P.a_c;
+                    const T w = P.c.r_c * fmaxf(fabsf(un + gc.cref), fabsf(un1 + gc.cref)) + P.c.a_c;
                     const T q = e / w;
                     Cc.es += (double)(q * q);
                     Cc.ec += 1;
@@ -590,7 +598,9 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
         }
     }
     if (ERR) block_partials(C[0].es + C[1].es, C[0].ec + C[1].ec, P.part_sum, P.part_cnt, bid, P.part_n, nblk);
-    // the step is counted by the wide pass, after the crowded cells
+    // the step is counted by the wide pass, after the crowded cells, where
+    // there can be any
+    if (P.count_step && !vec_crowds(g)) count_step_done(P.flag, nblk);
 }
 
 // The wide pass after a two-cell pass: every crowded cell recorded by the
@@ -600,7 +610,8 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
 // so the norm stays deterministic.  Blocks take the recorded entries in a
 // grid-stride loop; the last block to finish clears the record and, for a
 // pass that completes a fixed step, counts the step.  It runs after every
-// two-cell pass (with no entries it only does the bookkeeping).
+// two-cell pass of a problem that can have crowded cells (vec_crowds; with
+// no entries it only does the bookkeeping).
 constexpr int WIDE_FIX_BLOCKS = 152;
 
 // The recorded entries e = w, w + nw, ... of one two-cell pass.
@@ -642,12 +653,13 @@ __device__ __forceinline__ void wide_fix_entries(const Geom &g, const Pass<float
 }
 
 // After every block of the wide pass: clear the record and, for a pass
-// that completes a fixed step without a flag, count the step.
-__device__ __forceinline__ void wide_fix_close(const Pass<float> &P)
+// that completes a fixed step without a flag, count the step (passes without
+// crowded cells have counted it themselves).
+__device__ __forceinline__ void wide_fix_close(const Geom &g, const Pass<float> &P)
 {
     atomicExch(P.crowd, 0);
     atomicExch(P.crowd + 1, 0);
-    if (P.count_step && !pass_skipped(P.flag)) atomicAdd(P.flag + 1, 1);
+    if (P.count_step && vec_crowds(g) && !pass_skipped(P.flag)) atomicAdd(P.flag + 1, 1);
 }
 
 template <int DIM, int KC>
@@ -658,7 +670,7 @@ __device__ __forceinline__ void wide_fix_body(const Geom &g, const Pass<float> &
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(P.crowd + 1, 1) == (int)gridDim.x - 1) wide_fix_close(P);
+        if (atomicAdd(P.crowd + 1, 1) == (int)gridDim.x - 1) wide_fix_close(g, P);
     }
 }
 
@@ -718,7 +730,7 @@ vec_kernel_d(const __grid_constant__ Geom g, const Pass<float> *__restrict__ Pd,
 // Packed launches (batched serving): one launch runs the same pass kind
 // (dimension, K, signature) of several problems.  The blocks of problem k
 // are blocks bstart[k] .. bstart[k + 1] - 1 of the launch; each block finds
-// its problem by binary search, copies that problem's constants and pass
+// its problem, copies that problem's constants and pass
 // description into shared memory and runs the two-cell body on its tile, so
 // every problem computes exactly what its own launch would.
 // ---------------------------------------------------------------------------
@@ -730,15 +742,14 @@ struct VecInst {
     int nblk;                        // two-cell blocks of this problem
 };
 
-__device__ __forceinline__ int packed_find(const int *__restrict__ bstart, int n, int b)
+// Copies a struct into shared memory with the whole block.
+template <typename S>
+__device__ __forceinline__ void block_copy(S &dst, const S &src)
 {
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(bstart + mid) <= b) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
+    static_assert(sizeof(S) % 8 == 0, "copied in 8-byte words");
+    const unsigned long long *s = reinterpret_cast<const unsigned long long *>(&src);
+    unsigned long long *d = reinterpret_cast<unsigned long long *>(&dst);
+    for (int k = threadIdx.x; k < (int)(sizeof(S) / 8); k += blockDim.x) d[k] = s[k];
 }
 
 template <int DIM, int KC, unsigned SIG>
@@ -747,16 +758,19 @@ packed_kernel(const VecInst *__restrict__ tab, const int *__restrict__ bstart, i
 {
     __shared__ Geom gs;
     __shared__ Pass<float> Ps;
-    __shared__ int ks;
-    if (threadIdx.x == 0) {
-        const int k = packed_find(bstart, n, blockIdx.x);
-        ks = k;
-        gs = tab[k].g;
-        Ps = tab[k].P;
+    // the block's problem: the last k with bstart[k] <= block (prefix sums
+    // ascend), counted by the whole block with one round of loads per VBLOCK
+    // problems, then the description copied by the whole block (a thread-0
+    // binary search and copy took 16 us of a pass at 24 problems)
+    int k = -1;
+    for (int k0 = 0; k0 < n; k0 += VBLOCK) {
+        const int j = k0 + (int)threadIdx.x;
+        k += __syncthreads_count(j < n && __ldg(bstart + j) <= (int)blockIdx.x);
     }
-    __syncthreads();
-    const int k = ks;
     const VecInst &I = tab[k];
+    block_copy(gs, I.g);
+    block_copy(Ps, I.P);
+    __syncthreads();
     const int b = blockIdx.x - __ldg(bstart + k);
     const int tiles_x = (gs.nx + 2 * VTX - 1) / (2 * VTX), tiles_y = (gs.ny + VTY - 1) / VTY;
     vec_body<DIM, KC, SIG>(gs, Ps, I.A, I.B, I.L, I.ptype, b % tiles_x, (b / tiles_x) % tiles_y,
@@ -772,13 +786,14 @@ packed_wide_fix_kernel(const VecInst *__restrict__ tab, int n, int *done)
 {
     for (int k = 0; k < n; ++k) {
         const VecInst &I = tab[k];
+        if (!vec_crowds(I.g)) continue;
         wide_fix_entries<DIM, KC>(I.g, I.P, I.A, I.B, I.L, I.ptype, blockIdx.x, gridDim.x);
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(done, 1) == (int)gridDim.x - 1) {
-            for (int k = 0; k < n; ++k) wide_fix_close(tab[k].P);
+            for (int k = 0; k < n; ++k) wide_fix_close(tab[k].g, tab[k].P);
             atomicExch(done, 0);
         }
     }
