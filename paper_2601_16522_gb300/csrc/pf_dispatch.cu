@@ -43,10 +43,12 @@ int prepare_m32k1();
 
 template <>
 int launch_stage<double>(const Geom &g, const Pass<double> &P, cudaStream_t st, const double *A, const double *B,
-                         const double *L, const signed char *ptype, const TmaMaps *, int *nk)
+                         const double *L, const signed char *ptype, const TmaMaps *, int *nk,
+                         bool *kept)
 {
     bool done = false;
     if (nk) *nk = 1;
+    if (kept) *kept = false;
     // FP64 runs every pass through the generic instantiation
     int e = launch_f64(g, P, SIG_GENERIC, st, A, B, L, ptype, nullptr, &done);
     return done ? e : (int)cudaErrorInvalidValue;
@@ -54,10 +56,12 @@ int launch_stage<double>(const Geom &g, const Pass<double> &P, cudaStream_t st, 
 
 template <>
 int launch_stage<float>(const Geom &g, const Pass<float> &P, cudaStream_t st, const float *A, const float *B,
-                        const float *L, const signed char *ptype, const TmaMaps *tma, int *nk)
+                        const float *L, const signed char *ptype, const TmaMaps *tma, int *nk,
+                        bool *kept)
 {
     bool done = false;
     if (nk) *nk = 1;
+    if (kept) *kept = false;
     if (g.slots) {
         // slot storage: only the slot instantiations read the layout; a pass
         // kind without one is refused (cudaErrorInvalidValue)
@@ -85,6 +89,7 @@ int launch_stage<float>(const Geom &g, const Pass<float> &P, cudaStream_t st, co
                     : launch_v32k0(g, P, sig, st, A, B, L, ptype, &done);
         if (done) {
             if (nk) *nk = vec_crowds(g) ? 2 : 1;     // the pass and the wide pass of its crowded cells
+            if (kept) *kept = true;
             return e;
         }
     }

@@ -52,6 +52,67 @@ __global__ void pack_kernel(const double *__restrict__ phi, const double *__rest
     }
 }
 
+// pack_kernel for state vectors with segment words (pf_vec.cuh): one warp per
+// segment takes its cells lane and lane + 32 of every field (coalesced
+// whatever the alignment of phi) and votes the segment's words on the way, so
+// the words cost no pass of their own.
+template <typename T>
+__global__ void __launch_bounds__(256)
+pack_seg_kernel(const Geom g, const double *__restrict__ phi, const double *__restrict__ c, T *__restrict__ dst)
+{
+    const int lane = threadIdx.x & 31;
+    const long long q = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int tx = (g.nx + pfk::SEG_CELLS - 1) / pfk::SEG_CELLS;
+    if (q >= pfk::seg_count(g)) return;
+    const int row = (int)(q / tx), x0 = (int)(q - (long long)row * tx) * pfk::SEG_CELLS;
+    const int len = g.nx - x0 < pfk::SEG_CELLS ? g.nx - x0 : pfk::SEG_CELLS;
+    const long long i = (long long)row * g.nx + x0 + lane;
+    const bool h0 = lane < len, h1 = lane + 32 < len;
+    unsigned any = 0u, first = 0u, last = 0u;
+    const int nw = pfk::seg_words(g.N);
+    for (int w = 0; w < nw; ++w) {
+        const int n = g.N - 32 * w < 32 ? g.N - 32 * w : 32;
+#pragma unroll 8
+        for (int b = 0; b < n; ++b) {
+            const long long f = 32 * w + b;
+            T v0 = (T)0, v1 = (T)0;
+            if (h0) v0 = (T)phi[f * g.V + i];
+            if (h1) v1 = (T)phi[f * g.V + i + 32];
+            if (h0) dst[f * g.Vs + i] = v0;
+            if (h1) dst[f * g.Vs + i + 32] = v1;
+            const unsigned b0 = __ballot_sync(0xffffffffu, !pfk::zbits(v0)),
+                           b1 = __ballot_sync(0xffffffffu, !pfk::zbits(v1));
+            const unsigned long long m = ((unsigned long long)b1 << 32) | b0;
+            if (lane == w) {
+                if (m) any |= 1u << b;
+                if (m & 1ull) first |= 1u << b;
+                if ((m >> (len - 1)) & 1ull) last |= 1u << b;
+            }
+        }
+    }
+    if (lane < nw) {
+        pfk::seg_at(g, dst, (int)q, pfk::SEG_ANY)[lane] = any;
+        pfk::seg_at(g, dst, (int)q, pfk::SEG_FIRST)[lane] = first;
+        pfk::seg_at(g, dst, (int)q, pfk::SEG_LAST)[lane] = last;
+    }
+    if (g.K) {
+        if (h0) dst[g.N * g.Vs + i] = (T)(c[i] - g.cref);
+        if (h1) dst[g.N * g.Vs + i + 32] = (T)(c[i + 32] - g.cref);
+    }
+}
+
+// Segment words after the pointwise first stage (u1 = S(u + b1 F), F updated
+// in place): both outputs are +0 where u and F are.
+__global__ void seg_union_kernel(const unsigned *__restrict__ u, unsigned *__restrict__ f, unsigned *__restrict__ out,
+                                 long long n)
+{
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
+        const unsigned m = u[k] | f[k];
+        f[k] = m;
+        out[k] = m;
+    }
+}
+
 // engine layout -> ABI layout (phi and c as for pack_kernel; c may be null)
 template <typename T>
 __global__ void unpack_kernel(const T *__restrict__ src, double *__restrict__ phi, double *__restrict__ c, long long V,
@@ -546,6 +607,7 @@ struct pf_handle {
     cudaGraph_t dl_graph = nullptr;
     cudaGraphExec_t dl_exec = nullptr;
     int dl_integ = -1;
+    bool dl_kept = false;              // its passes write the segment words
     // reuse of F(u^{n+1}) as the next step's F(u^n) (PF_STEP_REUSE_RHS):
     // buffer rhs_buf holds the raw RHS of the state in buffer rhs_iu
     bool reuse_on = false, rhs_valid = false;
@@ -655,6 +717,21 @@ int invalidate_mask(pf_handle *h, const void *vecp)
                    cudaSuccess ? PF_OK : PF_EDEVICE;
 }
 
+// Segment words of a state vector (g.seg).
+unsigned *seg_words_of(const pf_handle *h, const void *vecp)
+{
+    return (unsigned *)((char *)const_cast<void *>(vecp) + (size_t)h->Vs * h->NP * h->esize);
+}
+
+// After a pass that wrote a state vector without its segment words: every
+// phase possibly nonzero everywhere.
+int invalidate_seg(pf_handle *h, const void *vecp)
+{
+    if (!h->g.seg || !vecp || buf_index(h, vecp) < 0) return PF_OK;
+    return cudaMemsetAsync(seg_words_of(h, vecp), 0xff, sizeof(unsigned) * (size_t)pfk::seg_vec_words(h->g),
+                           h->stream) == cudaSuccess ? PF_OK : PF_EDEVICE;
+}
+
 template <typename T>
 int run_pass(pf_handle *h, const Pass<T> &P0)
 {
@@ -707,10 +784,16 @@ int run_pass(pf_handle *h, const Pass<T> &P0)
         return prof_end(h);
     }
     int nk = 1;
+    bool kept = false;
     int e = pfk::launch_stage<T>(h->g, P, h->stream, (const T *)h->dA, (const T *)h->dB, (const T *)h->dL,
-                                 h->dptype, tmp, &nk);
+                                 h->dptype, tmp, &nk, &kept);
     h->launches += nk;
     if (e != 0) return PF_EDEVICE;
+    if (h->g.seg && !kept && P.mode != pfk::MODE_RHS) {
+        const void *outs[] = {P.mode == pfk::MODE_ERR ? nullptr : P.out, P.r0out, P.zout, P.out2};
+        for (const void *o : outs)
+            if ((st = invalidate_seg(h, o))) return st;
+    }
     if (h->masked && P.mode != pfk::MODE_RHS) {
         // a dense pass (generic kernel) wrote these vectors: their masks are stale
         const void *outs[] = {P.out, P.r0out, P.zout, P.out2};
@@ -1029,6 +1112,11 @@ int do_step(pf_handle *h, int integ, double dt, int s, const pf_tol *tol, bool w
             first_from_rhs_kernel<T><<<grid_for(h->V), 256, 0, h->stream>>>(B(U), B(ring[0]), B(r0), h->V, h->Vs,
                                                                              h->N, h->K, mt1 * dt, o2 ? 1 : 0, h->dflag);
         h->launches++;
+        if (h->g.seg)
+            seg_union_kernel<<<grid_for(pfk::seg_vec_words(h->g)), 256, 0, h->stream>>>(
+                seg_words_of(h, B(U)), seg_words_of(h, B(r0)), seg_words_of(h, B(ring[0])),
+                pfk::seg_vec_words(h->g));
+        h->launches += h->g.seg ? 1 : 0;
         if (cudaGetLastError() != cudaSuccess) return PF_EDEVICE;
         if ((st = prof_end(h))) return st;
         h->rhs_valid = false;
@@ -1485,6 +1573,7 @@ int build_devloop(pf_handle *h, int integ)
     h->dl_graph = top;
     h->dl_exec = exec;
     h->dl_integ = integ;
+    h->dl_kept = h->g.kvar == pfk::KVAR_TWO_CELL;
     return PF_OK;
 }
 
@@ -1556,6 +1645,9 @@ int devloop(pf_handle *h, int integ, double t_end, const pf_tol *tol, const pf_s
         if (cudaStreamSynchronize(h->stream) != cudaSuccess || !okc) st = st ? st : PF_EDEVICE;
     }
     if (o->trace_len) *o->trace_len = c.ntr;
+    if (!h->dl_kept)
+        for (int k = 0; k < NBUF; ++k)
+            if (invalidate_seg(h, h->buf[k])) st = st ? st : PF_EDEVICE;
     h->t = c.t;
     h->iu = c.iu;
     h->b = c.b;
@@ -1787,8 +1879,12 @@ int set_state_t(pf_handle *h, const double *phi_dev, const double *c_dev)
         if (cudaGetLastError() != cudaSuccess) return PF_EDEVICE;
         return check_flag(h);
     }
-    pack_kernel<T><<<grid_for(h->V * h->NP), 256, 0, h->stream>>>(phi_dev, c_dev, (T *)h->buf[h->iu], h->V, h->Vs,
-                                                                    h->N, h->NP, h->g.cref);
+    if (h->g.seg)
+        pack_seg_kernel<T><<<(unsigned)((pfk::seg_count(h->g) + 7) / 8), 256, 0, h->stream>>>(h->g, phi_dev, c_dev,
+                                                                                            (T *)h->buf[h->iu]);
+    else
+        pack_kernel<T><<<grid_for(h->V * h->NP), 256, 0, h->stream>>>(phi_dev, c_dev, (T *)h->buf[h->iu], h->V, h->Vs,
+                                                                        h->N, h->NP, h->g.cref);
     h->launches++;
     if (h->masked) {
         mask_kernel<<<grid_for(h->V), 256, 0, h->stream>>>((const float *)h->buf[h->iu], mask_plane(h, h->buf[h->iu]),
@@ -2095,8 +2191,10 @@ int pf_create(const pf_params *p, void *cuda_stream, pf_handle **out)
         h->masked = true;
         h->nw = (p->n_phases + 31) / 32;
     }
+    g.seg = h->prec == 32 && pfk::seg_eligible(g, slots, h->masked) ? 1 : 0;
     h->vec_bytes = slots ? sizeof(float) * (size_t)h->Vs * pfk::slot_planes(h->K)
                          : (size_t)h->Vs * NP * h->esize + sizeof(unsigned) * (size_t)h->Vs * h->nw;
+    if (g.seg) h->vec_bytes += sizeof(unsigned) * (size_t)pfk::seg_vec_words(g);
     bool ok = true;
     for (int k = 0; k < NBUF && ok; ++k) ok = dmalloc(h, &h->buf[k], h->vec_bytes);
     ok = ok && dmalloc(h, &h->dA, h->esize * N * N);
@@ -2149,6 +2247,7 @@ int pf_create(const pf_params *p, void *cuda_stream, pf_handle **out)
     }
     st |= cudaMemsetAsync(h->dflag, 0, PF_FLAG_BYTES, h->stream);
     if (h->dcrowd) st |= cudaMemsetAsync(h->dcrowd, 0, 2 * sizeof(int), h->stream);
+    for (int k = 0; k < NBUF; ++k) st |= invalidate_seg(h, h->buf[k]) == PF_OK ? 0 : 1;
     if (h->masked)
         for (int k = 0; k < NBUF; ++k)
             st |= cudaMemsetAsync(mask_plane(h, h->buf[k]), 0xff, sizeof(unsigned) * (size_t)h->Vs * h->nw,
@@ -2195,6 +2294,12 @@ int pf_footprint(const pf_params *p, long long *bytes)
     long long b = slots ? (long long)NBUF * pfk::slot_planes(p->has_conc ? 1 : 0) * Vs * 4   // slot vectors
                         : (long long)NBUF * NF * Vs * es;                                    // state vectors
     if (p->options & PF_OPT_MASKED) b += (long long)NBUF * ((p->n_phases + 31) / 32) * Vs * 4;   // occupancy words
+    if (!slots && p->precision == 32) {                   // segment words
+        pfk::Geom g{};
+        g.nx = p->nx; g.ny = p->ny; g.nz = p->nz; g.V = V; g.N = p->n_phases;
+        g.simplex = (p->options & PF_OPT_MOBILITY_SIMPLEX) ? pfk::SIMPLEX_MOBILITY : pfk::SIMPLEX_STANDARD;
+        if (pfk::seg_eligible(g, false, false)) b += (long long)NBUF * pfk::seg_vec_words(g) * 4;
+    }
     if (!slots) b += NF * V * 8;                           // ABI staging buffer (allocated on first set/get)
     b += 3LL * p->n_phases * p->n_phases * es + p->n_phases;   // coefficient tables, phase types
     if (!slots) b += 2LL * p->n_phases * p->n_phases * 8;  // FP64 A and B for the energy functional

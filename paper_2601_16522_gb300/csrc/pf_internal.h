@@ -12,10 +12,11 @@ namespace pfk {
 // (specialised FP32 hot passes) or the generic kernel.  Returns a cudaError_t.
 // tma: tensor maps of the pass's buffers for the TMA-staged FP32 kernels
 // (nullptr: plain loads).
-// *nk (may be null) receives the number of kernels the pass launched.
+// *nk (may be null) receives the number of kernels the pass launched, *kept
+// (may be null) whether it wrote the segment words of its output vectors.
 template <typename T>
 int launch_stage(const Geom &g, const Pass<T> &P, cudaStream_t st, const T *A, const T *B, const T *L,
-                 const signed char *ptype, const TmaMaps *tma, int *nk = nullptr);
+                 const signed char *ptype, const TmaMaps *tma, int *nk = nullptr, bool *kept = nullptr);
 
 // Kernels one pass of the device-driven loop launches (two-cell passes add
 // the wide pass of their crowded cells).

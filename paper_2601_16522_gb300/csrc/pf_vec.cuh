@@ -53,18 +53,6 @@ constexpr int VCELLS = 2 * VBLOCK;   // 256 cells per block
 #ifndef PF_VEC_MINB_LIGHT
 #define PF_VEC_MINB_LIGHT 7
 #endif
-// Phases ahead whose planes are prefetched into L2 (0: none).
-#ifndef PF_VEC_PREFETCH
-#define PF_VEC_PREFETCH 4
-#endif
-// ... for the passes with fewer pointwise streams
-#ifndef PF_VEC_PREFETCH_LIGHT
-#define PF_VEC_PREFETCH_LIGHT 0
-#endif
-// Register double buffering of the phase loads (1) or one phase at a time (0).
-#ifndef PF_VEC_DB
-#define PF_VEC_DB 1
-#endif
 
 // Blocks of the x-y plane of the two-cell kernels (one z plane per block).
 __host__ __device__ inline long long vec_tiles(const Geom &g)
@@ -130,6 +118,68 @@ __device__ __forceinline__ float fmin3(float a, float b, float c)
     return r;
 }
 
+// ---------------------------------------------------------------------------
+// Segment words.  A dense FP32 state vector is followed (after its NF planes)
+// by a small record per segment, 64 consecutive cells of one row: for every
+// phase one bit that is clear only where the phase is exactly +0 in all 64
+// cells, and the same for the segment's first and last cell alone (what the
+// neighbouring segments' x differences read).  A warp of a two-cell pass owns
+// one segment: it visits only the phases that are set in a word its results
+// depend on (its own, the y/z neighbours', the facing edge cells' and those of
+// the pointwise inputs); every other phase has inputs that are all +0, whose
+// stage value is +0, and is stored only where the output's old word says that
+// it still holds something else.  Results are those of visiting every phase,
+// bit for bit.  At 256^3 x 32 grains a segment sees about 3 of the 32 phases;
+// the words cost 12 bytes per 64 cells and vector.
+// Problems of up to SEG_MIN_PHASES phases keep no words (g.seg = 0): their
+// phases are present nearly everywhere, and the loads of the words would only
+// lengthen each warp's chain.
+// ---------------------------------------------------------------------------
+constexpr int SEG_CELLS = 2 * VTX;
+constexpr int SEG_MIN_PHASES = 4;
+enum { SEG_ANY = 0, SEG_FIRST = 1, SEG_LAST = 2, SEG_KINDS = 3 };
+
+__host__ __device__ inline int seg_words(int N) { return (N + 31) / 32; }
+__host__ __device__ inline long long seg_count(const Geom &g)
+{
+    return (long long)((g.nx + SEG_CELLS - 1) / SEG_CELLS) * g.ny * g.nz;
+}
+// Whether the state vectors of a problem carry segment words (dense FP32
+// storage; slots and masked are the storage options).
+__host__ __device__ inline bool seg_eligible(const Geom &g, bool slots, bool masked)
+{
+    return !slots && !masked && g.simplex == SIMPLEX_STANDARD && vec_eligible(g) && g.N > SEG_MIN_PHASES;
+}
+// Words of one state vector.
+__host__ __device__ inline long long seg_vec_words(const Geom &g) { return seg_count(g) * SEG_KINDS * seg_words(g.N); }
+
+// Word `kind` (base: + w) of segment q of a state vector.
+template <typename T>
+__device__ __forceinline__ unsigned *seg_at(const Geom &g, const T *vec, int q, int kind)
+{
+    return const_cast<unsigned *>(reinterpret_cast<const unsigned *>(vec + (long long)g.NF * g.Vs)) +
+           ((long long)q * SEG_KINDS + kind) * seg_words(g.N);
+}
+
+// Adds the phases of one cell, rewritten by the wide pass, to its segment's
+// words.
+__device__ __forceinline__ void seg_add_cell(const Geom &g, const float *vec, int x, int y, int z)
+{
+    const int tx = (g.nx + SEG_CELLS - 1) / SEG_CELLS;
+    const int q = (z * g.ny + y) * tx + x / SEG_CELLS;
+    const bool first = x % SEG_CELLS == 0, last = x % SEG_CELLS == SEG_CELLS - 1 || x == g.nx - 1;
+    const long long i = ((long long)z * g.ny + y) * g.nx + x;
+    for (int w = 0; w < seg_words(g.N); ++w) {
+        unsigned m = 0u;
+        for (int b = 0; b < 32 && 32 * w + b < g.N; ++b)
+            if (__float_as_uint(vec[(long long)(32 * w + b) * g.Vs + i]) != 0u) m |= 1u << b;
+        if (!m) continue;
+        atomicOr(seg_at(g, vec, q, SEG_ANY) + w, m);
+        if (first) atomicOr(seg_at(g, vec, q, SEG_FIRST) + w, m);
+        if (last) atomicOr(seg_at(g, vec, q, SEG_LAST) + w, m);
+    }
+}
+
 // Loads of one phase for the thread's two cells.
 struct VPhase {
     float2 c, ym, yp, zm, zp;  // stencil input at the pair and its y/z neighbours
@@ -161,7 +211,10 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
     constexpr bool HR0 = (SIG & SIG_R0IN) != 0 || ERR;
     constexpr bool R0OUT = (SIG & SIG_R0OUT) != 0;
     constexpr bool PROJ = (SIG & SIG_PROJECT) != 0;
+    constexpr unsigned ALL = 0xffffffffu;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
+    __shared__ unsigned visited[VTY][4];   // the phases each warp visits (N <= 128)
+    __shared__ unsigned fixed[VTY][4];     // phases not listed whose F the first-stage fix replaced
     if (pass_skipped(P.flag)) return;
     constexpr int VACT = vec_act<SIG>();   // nontrivial phases per cell in the shared-memory list
     VecSmem<VACT> &S = *reinterpret_cast<VecSmem<VACT> *>(smem_raw);
@@ -183,9 +236,10 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
     bool crowd[2] = {false, false};
     if (y < g.ny) {   // warp-uniform (a warp is one row)
         const bool here = x < g.nx;
-        const int i = (z * g.ny + y) * g.nx + x;
+        const int row = z * g.ny + y;
+        const int i = row * g.nx + x;
         // lanes past nx load the last pair of their row (in bounds, unused)
-        const int il = here ? i : (z * g.ny + y) * g.nx + (g.nx - 2);
+        const int il = here ? i : row * g.nx + (g.nx - 2);
         // y / z neighbour offsets (a zero-gradient ghost is the cell itself)
         long long off64[6];
         int ghost[6];
@@ -207,6 +261,23 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
         const T ib1 = P.c.ib1;
         const T dt = P.c.dt, rph = P.c.r_phi, aph = P.c.a_phi;
 
+        // segments: own, y/z neighbours, left and right along the row
+        const bool seg = g.seg != 0;
+        const int nw = seg_words(N);
+        const int q0 = row * tiles_x + bx;
+        const int srow = tiles_x;
+        const int qym = q0 + (y > 0 ? -srow : (g.bc_phi[2] == BC_PERIODIC ? (g.ny - 1) * srow : 0));
+        const int qyp = q0 + (y < g.ny - 1 ? srow : (g.bc_phi[3] == BC_PERIODIC ? -(g.ny - 1) * srow : 0));
+        const int splane = srow * g.ny;
+        const int qzm = DIM == 3 ? q0 + (z > 0 ? -splane : (g.bc_phi[4] == BC_PERIODIC ? (g.nz - 1) * splane : 0)) : q0;
+        const int qzp = DIM == 3 ? q0 + (z < g.nz - 1 ? splane : (g.bc_phi[5] == BC_PERIODIC ? -(g.nz - 1) * splane : 0))
+                                 : q0;
+        const int ql = bx > 0 ? q0 - 1 : (g.bc_phi[0] == BC_PERIODIC ? q0 + tiles_x - 1 : -1);
+        const int qr = bx < tiles_x - 1 ? q0 + 1 : (g.bc_phi[1] == BC_PERIODIC ? q0 - (tiles_x - 1) : -1);
+        const int lastlane = min(31, (g.nx - 2 - bx * (2 * VTX)) / 2);   // lane of the segment's last cell
+        // words of the output's segment, word w held by lane w
+        unsigned w_any = 0u, w_first = 0u, w_last = 0u, w_r0 = 0u;
+
         // concentration: per chemical type, phase sums of the two cells, of
         // their y/z neighbours and of the x edge cells
         T Ph[2][2], Pn[2][4][2], Pe[2][2];
@@ -221,37 +292,37 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
         // bases below are the same for every thread (uniform)
         const int oc = il, oym_ = il + oym, oyp_ = il + oyp, ozm_ = il + ozm, ozp_ = il + ozp;
         const int oel = il + lofs, oer = il + rofs;
-        auto fetch = [&](int a, VPhase &q) {
-            const long long pb = (long long)a * Vs;
+        // which of a phase's inputs can be nonzero (uniform words)
+        unsigned mS = ALL, mP0 = ALL, mP2 = ALL, mR0 = ALL, mO = ALL, mR = ALL;
+        auto fetch = [&](int bit, long long pb, VPhase &q) {
             const float *b = P.in + pb;
-            constexpr int PD = (HP0 && HP2) ? PF_VEC_PREFETCH : PF_VEC_PREFETCH_LIGHT;
-            if (PD > 0 && a + PD < N) {
-                const long long pa = pb + (long long)PD * Vs;
-                prefetch_l2(P.in + pa + oc);
-                if (HP0) prefetch_l2(P.p0 + pa + oc);
-                if (HP2) prefetch_l2(P.p2 + pa + oc);
-                if (HR0) prefetch_l2(P.r0in + pa + oc);
+            const float2 zero = make_float2(0.f, 0.f);
+            if ((mS >> bit) & 1u) {
+                q.c = ldg2(b + oc);
+                q.ym = ldg2(b + oym_);
+                q.yp = ldg2(b + oyp_);
+                if (DIM == 3) {
+                    q.zm = ldg2(b + ozm_);
+                    q.zp = ldg2(b + ozp_);
+                }
+                if (lneed) q.el = __ldg(b + oel);
+                if (rneed) q.er = __ldg(b + oer);
+            } else {
+                q.c = q.ym = q.yp = q.zm = q.zp = zero;
+                q.el = q.er = 0.f;
             }
-            q.c = ldg2(b + oc);
-            q.ym = ldg2(b + oym_);
-            q.yp = ldg2(b + oyp_);
-            if (DIM == 3) {
-                q.zm = ldg2(b + ozm_);
-                q.zp = ldg2(b + ozp_);
-            }
-            if (HP0) q.p0 = ld_stream2(P.p0 + pb + oc);
-            if (HP2) q.p2 = ld_stream2(P.p2 + pb + oc);
-            if (HR0) q.r0 = ld_stream2(P.r0in + pb + oc);
-            if (lneed) q.el = __ldg(b + oel);
-            if (rneed) q.er = __ldg(b + oer);
+            if (HP0) q.p0 = ((mP0 >> bit) & 1u) ? ld_stream2(P.p0 + pb + oc) : zero;
+            if (HP2) q.p2 = ((mP2 >> bit) & 1u) ? ld_stream2(P.p2 + pb + oc) : zero;
+            if (HR0) q.r0 = ((mR0 >> bit) & 1u) ? ld_stream2(P.r0in + pb + oc) : zero;
         };
 
-        // one phase at one cell: activity, list entry, stage value (returned)
+        // one phase at one cell: activity, list entry, stage value (returned);
+        // *occ: not listed and not +0
         auto cell_phase = [&](VCell &Cc, int slot, int a, T v, T xl, T xr, T ym, T yp, T zm, T zp, T p0v, T p2v,
-                              T r0v) -> T {
-            // every input +0 (most phases of most cells): the phase is not
-            // nontrivial, its stage value is exactly +0, it adds nothing to the
-            // sum, the count or the error -- the result of the steps below
+                              T r0v, bool *occ) -> T {
+            // every input +0: the phase is not nontrivial, its stage value is
+            // exactly +0, it adds nothing to the sum, the count or the error --
+            // the result of the steps below
             unsigned bits = __float_as_uint(v) | __float_as_uint(xl) | __float_as_uint(xr) | __float_as_uint(ym) |
                             __float_as_uint(yp);
             if (DIM == 3) bits |= __float_as_uint(zm) | __float_as_uint(zp);
@@ -299,14 +370,16 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                 if (acc >= (T)1 && acc > Cc.best) { Cc.best = acc; Cc.bestid = a; }
                 Cc.ssum = Cc.ssum + acc;
                 if (acc != (T)0) Cc.nzcnt++;
+                *occ = __float_as_uint(acc) != 0u;
             }
             return acc;
         };
 
         // ---- the sweep over the phases ---------------------------------------
-        auto process = [&](int a, const VPhase &q) {
-            const float sl = __shfl_up_sync(0xffffffffu, q.c.y, 1);
-            const float sr = __shfl_down_sync(0xffffffffu, q.c.x, 1);
+        auto process = [&](int w, int bit, long long pb, const VPhase &q) {
+            const int a = 32 * w + bit;
+            const float sl = __shfl_up_sync(ALL, q.c.y, 1);
+            const float sr = __shfl_down_sync(ALL, q.c.x, 1);
             const T left = lsh ? sl : (lself ? q.c.x : q.el);
             const T right = rsh ? sr : (rself ? q.c.y : q.er);
             const T zm0 = DIM == 3 ? q.zm.x : (T)0, zm1 = DIM == 3 ? q.zm.y : (T)0;
@@ -314,13 +387,16 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
             const T p00 = HP0 ? q.p0.x : (T)0, p01 = HP0 ? q.p0.y : (T)0;
             const T p20 = HP2 ? q.p2.x : (T)0, p21 = HP2 ? q.p2.y : (T)0;
             const T r00 = HR0 ? q.r0.x : (T)0, r01 = HR0 ? q.r0.y : (T)0;
+            bool occ0 = false, occ1 = false;
             if (here) {
-                const T w0 = cell_phase(C[0], tid, a, q.c.x, left, q.c.y, q.ym.x, q.yp.x, zm0, zp0, p00, p20, r00);
+                const T w0 = cell_phase(C[0], tid, a, q.c.x, left, q.c.y, q.ym.x, q.yp.x, zm0, zp0, p00, p20, r00,
+                                        &occ0);
                 const T w1 = cell_phase(C[1], VBLOCK + tid, a, q.c.y, q.c.x, right, q.ym.y, q.yp.y, zm1, zp1, p01,
-                                        p21, r01);
-                const long long pb = (long long)a * Vs;
+                                        p21, r01, &occ1);
                 if (!ERR) st2(P.out + pb + i, w0, w1);
-                if (R0OUT) st2(P.r0out + pb + i, (T)0, (T)0);   // listed phases get theirs below
+                // listed phases get their RHS below; where the word was clear
+                // the plane holds zero already
+                if (R0OUT && ((mR >> bit) & 1u)) st2(P.r0out + pb + i, (T)0, (T)0);
                 if (KC) {
                     const int t = ptype[a];
                     // per-type sums: own cells, y/z neighbours, edge cells
@@ -336,29 +412,85 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                     if (rneed) Pe[1][t] += q.er;
                 }
             }
-        };
-        // two phases per iteration: the loads of the next phase are in flight
-        // while the current one is processed, without register copies
-        if (PF_VEC_DB) {
-            VPhase qa, qb;
-            fetch(0, qa);
-            int a = 0;
-#pragma unroll 1
-            for (; a + 1 < N; a += 2) {
-                fetch(a + 1, qb);
-                process(a, qa);
-                if (a + 2 < N) fetch(a + 2, qa);
-                process(a + 1, qb);
+            if (!ERR && seg) {
+                const unsigned b0 = __ballot_sync(ALL, occ0), b1 = __ballot_sync(ALL, occ1);
+                if (lane == w) {
+                    const unsigned m = 1u << bit;
+                    if (b0 | b1) w_any |= m;
+                    if (b0 & 1u) w_first |= m;
+                    if ((b1 >> lastlane) & 1u) w_last |= m;
+                }
             }
-            if (a < N) process(a, qa);
-        } else {
-#pragma unroll 1
-            for (int a = 0; a < N; ++a) {
-                VPhase q;
-                fetch(a, q);
-                process(a, q);
+        };
+        for (int w = 0; w < nw; ++w) {
+            const unsigned full = word_bits(N, w);
+            unsigned U = full;
+            if (seg) {
+                auto word = [&](const float *v, int q, int kind) { return __ldg(seg_at(g, v, q, kind) + w); };
+                unsigned s = word(P.in, q0, SEG_ANY) | word(P.in, qym, SEG_ANY) | word(P.in, qyp, SEG_ANY);
+                if (DIM == 3) s |= word(P.in, qzm, SEG_ANY) | word(P.in, qzp, SEG_ANY);
+                if (ql >= 0) s |= word(P.in, ql, SEG_LAST);
+                if (qr >= 0) s |= word(P.in, qr, SEG_FIRST);
+                const unsigned p0w = HP0 ? word(P.p0, q0, SEG_ANY) : 0u;
+                const unsigned p2w = HP2 ? word(P.p2, q0, SEG_ANY) : 0u;
+                const unsigned r0w = HR0 ? word(P.r0in, q0, SEG_ANY) : 0u;
+                // the same in every lane; the reduction puts them into uniform
+                // registers, so the loop below and its addresses are uniform
+                mS = __reduce_or_sync(ALL, s);
+                if (HP0) mP0 = __reduce_or_sync(ALL, p0w);
+                if (HP2) mP2 = __reduce_or_sync(ALL, p2w);
+                if (HR0) mR0 = __reduce_or_sync(ALL, r0w);
+                if (!ERR) mO = __reduce_or_sync(ALL, seg_at(g, P.out, q0, SEG_ANY)[w]);
+                if (R0OUT) mR = __reduce_or_sync(ALL, seg_at(g, P.r0out, q0, SEG_ANY)[w]);
+                U = mS;
+                if (HP0) U |= mP0;
+                if (HP2) U |= mP2;
+                if (HR0) U |= mR0;
+                U &= full;
+                // phases not visited: +0, stored where the output holds another value
+                if (here) {
+                    if (!ERR)
+                        for (unsigned m = mO & full & ~U; m; m &= m - 1u)
+                            st2(P.out + (long long)(32 * w + __ffs(m) - 1) * Vs + i, (T)0, (T)0);
+                    if (R0OUT)
+                        for (unsigned m = mR & full & ~U; m; m &= m - 1u)
+                            st2(P.r0out + (long long)(32 * w + __ffs(m) - 1) * Vs + i, (T)0, (T)0);
+                }
+            }
+            if (lane == 0) {
+                visited[ty][w] = U;
+                if (R0OUT) fixed[ty][w] = 0u;
+            }
+            // two phases per iteration: the loads of the next phase are in flight
+            // while the current one is processed, without register copies
+            unsigned m = U;
+            if (m) {
+                VPhase qa, qb;
+                int a = __ffs(m) - 1, b;
+                m &= m - 1u;
+                long long pa = (long long)(32 * w + a) * Vs, pb = 0;
+                fetch(a, pa, qa);
+                for (;;) {
+                    b = __ffs(m) - 1;
+                    if (b >= 0) {
+                        m &= m - 1u;
+                        pb = (long long)(32 * w + b) * Vs;
+                        fetch(b, pb, qb);
+                    }
+                    process(w, a, pa, qa);
+                    if (b < 0) break;
+                    a = __ffs(m) - 1;
+                    if (a >= 0) {
+                        m &= m - 1u;
+                        pa = (long long)(32 * w + a) * Vs;
+                        fetch(a, pa, qa);
+                    }
+                    process(w, b, pb, qb);
+                    if (a < 0) break;
+                }
             }
         }
+        __syncwarp();
 
         // ---- concentration: mu of the cells and their neighbours, c RHS ------
         T mu[2] = {(T)0, (T)0}, rc[2] = {(T)0, (T)0}, cc[2] = {(T)0, (T)0};
@@ -493,11 +625,10 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
         }
 
         // ---- projection, final values, concentration ------------------------
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
+        auto finish = [&](int c) {
             VCell &Cc = C[c];
             const int slot = c * VBLOCK + tid;
-            if (!here || crowd[c]) continue;
+            if (!here || crowd[c]) return;
             const int nz = Cc.nz;
             if (ERR) {
                 Cc.ec += (Cc.nc > 0 ? Cc.nc : 2);
@@ -511,7 +642,7 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                     Cc.ec += 1;
                     if (R0OUT) P.r0out[o] = rc[c];
                 }
-                continue;
+                return;
             }
             bool rewrite = false;     // inactive nonzero entries need their final value
             if (PROJ) {
@@ -542,6 +673,7 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                 T w = S.val[k][slot];
                 if (PROJ) w = (Cc.bestid >= 0) ? ((a == Cc.bestid) ? (T)1 : (T)0) : w * inv;
                 P.out[fo] = w;
+                S.val[k][slot] = w;
                 if (R0OUT) {
                     T r = S.lap[k][slot];
                     if (fix) r = (w - S.cen[k][slot]) * ib1;
@@ -552,15 +684,20 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
             // bulk cells): the >= 1 rule or the normalisation
             if (rewrite) {
                 int kk = 0;
-                for (int a = 0; a < N; ++a) {
-                    if (kk < nz && S.id[kk][slot] == a) { kk++; continue; }
-                    const long long fo = (long long)a * Vs + i + c;
-                    const T o = P.out[fo];
-                    if (o == (T)0) continue;
-                    const T w = (Cc.bestid >= 0) ? ((a == Cc.bestid) ? (T)1 : (T)0) : o * inv;
-                    P.out[fo] = w;
-                    if (fix) P.r0out[fo] = (w - __ldg(P.in + fo)) * ib1;
-                }
+                for (int wd = 0; wd < nw; ++wd)
+                    for (unsigned m = visited[ty][wd]; m; m &= m - 1u) {
+                        const int a = 32 * wd + __ffs(m) - 1;
+                        if (kk < nz && S.id[kk][slot] == a) { kk++; continue; }
+                        const long long fo = (long long)a * Vs + i + c;
+                        const T o = P.out[fo];
+                        if (o == (T)0) continue;
+                        const T w = (Cc.bestid >= 0) ? ((a == Cc.bestid) ? (T)1 : (T)0) : o * inv;
+                        P.out[fo] = w;
+                        if (fix) {
+                            P.r0out[fo] = (w - __ldg(P.in + fo)) * ib1;
+                            if (seg) atomicOr(&fixed[ty][wd], 1u << (a & 31));
+                        }
+                    }
             }
             if (KC) {
                 const long long o = (long long)N * Vs + i + c;
@@ -573,6 +710,49 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                 if (!isfinite(acc)) raise_flag(P.flag, FLAG_NONFINITE);
                 if (R0OUT) P.r0out[o] = rc[c];
                 P.out[o] = acc;
+            }
+        };
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            finish(c);
+            if (ERR ? !R0OUT : false) continue;
+            if (!seg) continue;
+            // the listed phases' part of the output words
+            const int slot = c * VBLOCK + tid;
+            const int nz = here && !crowd[c] ? C[c].nz : 0;
+            for (int w = 0; w < nw; ++w) {
+                unsigned mv = 0u, ml = 0u;
+                for (int k = 0; k < nz; ++k) {
+                    const int a = S.id[k][slot];
+                    if (nw > 1 && (a >> 5) != w) continue;
+                    ml |= 1u << (a & 31);
+                    if (!ERR && __float_as_uint(S.val[k][slot]) != 0u) mv |= 1u << (a & 31);
+                }
+                if (!ERR) {
+                    const unsigned r = __reduce_or_sync(ALL, mv), e = __shfl_sync(ALL, mv, c == 0 ? 0 : lastlane);
+                    if (lane == w) {
+                        w_any |= r;
+                        if (c == 0) w_first |= e;
+                        else w_last |= e;
+                    }
+                }
+                if (R0OUT) {
+                    const unsigned r = __reduce_or_sync(ALL, ml);
+                    if (lane == w) w_r0 |= r;
+                }
+            }
+        }
+        __syncwarp();
+        if (seg && lane < nw) {
+            if (!ERR) {
+                seg_at(g, P.out, q0, SEG_ANY)[lane] = w_any;
+                seg_at(g, P.out, q0, SEG_FIRST)[lane] = w_first;
+                seg_at(g, P.out, q0, SEG_LAST)[lane] = w_last;
+            }
+            // F is read at its own cell only: its edge words need not be sharp
+            if (R0OUT && P.r0out) {
+                const unsigned r = w_r0 | fixed[ty][lane];
+                for (int k = 0; k < SEG_KINDS; ++k) seg_at(g, P.r0out, q0, k)[lane] = r;
             }
         }
     }
@@ -635,6 +815,10 @@ __device__ __forceinline__ void wide_fix_entries(const Geom &g, const Pass<float
             const int bx = b % tiles_x, by = (b / tiles_x) % tiles_y, bz = b / (tiles_x * tiles_y);
             const int x = bx * (2 * VTX) + (tid % (2 * VTX)), y = by * VTY + tid / (2 * VTX);
             wide_cell<float, DIM, KC>(&g, &P, tabA, tabB, tabL, ptype, x, y, bz, &es, &ec);
+            if (g.seg) {
+                if (P.mode == MODE_STAGE) seg_add_cell(g, P.out, x, y, bz);
+                if (P.r0out) seg_add_cell(g, P.r0out, x, y, bz);
+            }
         }
         if (P.mode == MODE_ERR) {
             rs[tid] = es;
