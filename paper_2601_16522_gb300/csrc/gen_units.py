@@ -2,7 +2,8 @@
 after changing a kernel template's parameters or the set of pass
 signatures; the written files are committed, and build.py compiles them).
 
-pf_stage_f64.cu      FP64: the generic stage kernel, 2D/3D, K = 0/1
+pf_stage_f64.cu      FP64: dbl_kernel (8 or 2 rows a block), 2D/3D, K = 0/1, and
+                     the generic stage kernel for the mobility-weighted projection
 pf_stage_f32k{0,1}   FP32, K fixed: big_kernel (32 < N <= 250), tma_kernel and
                      fast_kernel (N <= 32, NMAX 4 or 32) per pass signature
                      (fast_kernel also for the error sweep that keeps its RHS),
@@ -34,6 +35,25 @@ SSP_SIGS = ["SIG_O2 | SIG_PROJECT", "SIG_Z | SIG_PROJECT", "SIG_Z | SIG_O2 | SIG
 # passes of the device-driven adaptive RKL steps: stage 1, RKL2 body, RKL1
 # body, error sweep (descriptor-driven kernels)
 DSIGS = ["SIG_R0OUT | SIG_PROJECT", "SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT", "SIG_P2 | SIG_PROJECT", "SIG_ERR"]
+
+
+def dbl_launch(kernel, arg, prep):
+    """The FP64 passes with the standard projection (pf_dbl.cuh)."""
+    L = ["    if (g.simplex == SIMPLEX_STANDARD) {",
+         "        const int rows = dbl_rows(g);",
+         "        const dim3 dgrid((g.nx + DBL_TX - 1) / DBL_TX, (g.ny + rows - 1) / rows, g.nz);"]
+    for d in (2, 3):
+        for k in (0, 1):
+            for r in (2, 8):
+                L.append("        if (g.dim == %d && g.K == %d && rows == %d) {" % (d, k, r))
+                L.append("            %s<%d, %d, %d><<<dgrid, DBL_TX * %d, sizeof(DblSmem<%d>), st>>>(g, %s, A, B, L, ptype);"
+                         % (kernel, d, k, r, r, r, arg))
+                L.append("            return (int)cudaGetLastError();")
+                L.append("        }")
+                prep.append("    if (cudaFuncSetAttribute(%s<%d, %d, %d>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DblSmem<%d>)) != cudaSuccess) return -1;"
+                            % (kernel, d, k, r, r))
+    L.append("    }")
+    return L
 
 
 def unit(T, kcs, fast, fname):
@@ -91,6 +111,8 @@ def unit(T, kcs, fast, fname):
                     prep.append("    if (cudaFuncSetAttribute(fast_kernel<%d, %d, %s, %d>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf) != cudaSuccess) return -1;" % (d, kc, sg, nmax))
             L.append("        }")
         L.append("    }")
+    if not fast:
+        L += dbl_launch("dbl_kernel", "P", prep)
     L.append("    const size_t sm = sizeof(Smem<%s>);" % T)
     for d in (2, 3):
         for k in kcs:
@@ -126,6 +148,7 @@ def unit(T, kcs, fast, fname):
             L.append("        }")
         L.append("    }")
     else:
+        L += dbl_launch("dbl_kernel_d", "dP", prep)
         L.append("    const size_t sm = sizeof(Smem<%s>);" % T)
         for d in (2, 3):
             for k in kcs:

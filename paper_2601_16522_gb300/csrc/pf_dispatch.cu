@@ -49,8 +49,11 @@ int launch_stage<double>(const Geom &g, const Pass<double> &P, cudaStream_t st, 
     bool done = false;
     if (nk) *nk = 1;
     if (kept) *kept = false;
-    // FP64 runs every pass through the generic instantiation
+    // FP64 runs every pass through one kernel (options read at run time): the
+    // pass of pf_dbl.cuh, or the generic body for the mobility-weighted
+    // projection
     int e = launch_f64(g, P, SIG_GENERIC, st, A, B, L, ptype, nullptr, &done);
+    if (kept) *kept = g.simplex == SIMPLEX_STANDARD;
     return done ? e : (int)cudaErrorInvalidValue;
 }
 

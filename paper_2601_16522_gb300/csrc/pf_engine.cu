@@ -62,10 +62,10 @@ pack_seg_kernel(const Geom g, const double *__restrict__ phi, const double *__re
 {
     const int lane = threadIdx.x & 31;
     const long long q = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int tx = (g.nx + pfk::SEG_CELLS - 1) / pfk::SEG_CELLS;
+    const int tx = (g.nx + g.segc - 1) / g.segc;
     if (q >= pfk::seg_count(g)) return;
-    const int row = (int)(q / tx), x0 = (int)(q - (long long)row * tx) * pfk::SEG_CELLS;
-    const int len = g.nx - x0 < pfk::SEG_CELLS ? g.nx - x0 : pfk::SEG_CELLS;
+    const int row = (int)(q / tx), x0 = (int)(q - (long long)row * tx) * g.segc;
+    const int len = g.nx - x0 < g.segc ? g.nx - x0 : g.segc;
     const long long i = (long long)row * g.nx + x0 + lane;
     const bool h0 = lane < len, h1 = lane + 32 < len;
     unsigned any = 0u, first = 0u, last = 0u;
@@ -1573,7 +1573,7 @@ int build_devloop(pf_handle *h, int integ)
     h->dl_graph = top;
     h->dl_exec = exec;
     h->dl_integ = integ;
-    h->dl_kept = h->g.kvar == pfk::KVAR_TWO_CELL;
+    h->dl_kept = h->prec == 64 || h->g.kvar == pfk::KVAR_TWO_CELL;
     return PF_OK;
 }
 
@@ -2178,7 +2178,8 @@ int pf_create(const pf_params *p, void *cuda_stream, pf_handle **out)
     if (bps <= 0) { delete h; return PF_EINVAL; }
     if ((long long)g.tiles_x * g.tiles_y * p->nz > 0x7fffffffLL || p->nz > 65535) { delete h; return PF_EINVAL; }
     // error partials: one per block of the largest tiling an error pass may use
-    h->grid = (int)std::max((long long)g.tiles_x * g.tiles_y, pfk::vec_tiles(g)) * p->nz;
+    h->grid = (int)std::max((long long)g.tiles_x * g.tiles_y, h->prec == 64 ? pfk::dbl_tiles(g) : pfk::vec_tiles(g)) *
+              p->nz;
     h->tot_blocks = (int)((h->V + 4095) / 4096 < 1024 ? (h->V + 4095) / 4096 : 1024);
     if (h->tot_blocks < 1) h->tot_blocks = 1;
 
@@ -2191,7 +2192,8 @@ int pf_create(const pf_params *p, void *cuda_stream, pf_handle **out)
         h->masked = true;
         h->nw = (p->n_phases + 31) / 32;
     }
-    g.seg = h->prec == 32 && pfk::seg_eligible(g, slots, h->masked) ? 1 : 0;
+    g.segc = pfk::seg_length(h->prec);
+    g.seg = pfk::seg_eligible(g, h->prec, slots, h->masked) ? 1 : 0;
     h->vec_bytes = slots ? sizeof(float) * (size_t)h->Vs * pfk::slot_planes(h->K)
                          : (size_t)h->Vs * NP * h->esize + sizeof(unsigned) * (size_t)h->Vs * h->nw;
     if (g.seg) h->vec_bytes += sizeof(unsigned) * (size_t)pfk::seg_vec_words(g);
@@ -2294,11 +2296,12 @@ int pf_footprint(const pf_params *p, long long *bytes)
     long long b = slots ? (long long)NBUF * pfk::slot_planes(p->has_conc ? 1 : 0) * Vs * 4   // slot vectors
                         : (long long)NBUF * NF * Vs * es;                                    // state vectors
     if (p->options & PF_OPT_MASKED) b += (long long)NBUF * ((p->n_phases + 31) / 32) * Vs * 4;   // occupancy words
-    if (!slots && p->precision == 32) {                   // segment words
+    if (!slots) {                                          // segment words
         pfk::Geom g{};
         g.nx = p->nx; g.ny = p->ny; g.nz = p->nz; g.V = V; g.N = p->n_phases;
+        g.segc = pfk::seg_length(p->precision);
         g.simplex = (p->options & PF_OPT_MOBILITY_SIMPLEX) ? pfk::SIMPLEX_MOBILITY : pfk::SIMPLEX_STANDARD;
-        if (pfk::seg_eligible(g, false, false)) b += (long long)NBUF * pfk::seg_vec_words(g) * 4;
+        if (pfk::seg_eligible(g, p->precision, false, false)) b += (long long)NBUF * pfk::seg_vec_words(g) * 4;
     }
     if (!slots) b += NF * V * 8;                           // ABI staging buffer (allocated on first set/get)
     b += 3LL * p->n_phases * p->n_phases * es + p->n_phases;   // coefficient tables, phase types

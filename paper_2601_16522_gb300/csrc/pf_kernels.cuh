@@ -74,7 +74,8 @@ struct Geom : GeomConst<double> {
     int kvar;                           // FP32 dense passes: KVAR_TWO_CELL or KVAR_ONE_CELL
     int simplex;                        // projection S: SIMPLEX_STANDARD or SIMPLEX_MOBILITY
     int slots;                          // 1: per-cell phase slots (FP32; see pf_slots.cuh)
-    int seg;                            // 1: state vectors carry segment words (see pf_vec.cuh)
+    int seg, segc;                      // 1: state vectors carry segment words (see pf_vec.cuh);
+                                        // cells of a segment
     int uni;                            // slot passes: 1 if every off-diagonal entry of each
     float uA, uB, uL;                   // FP32 table A, B, L is the same value (these), which
                                         // the pairwise sums then use instead of gathers

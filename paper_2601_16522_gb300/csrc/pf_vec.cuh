@@ -119,10 +119,10 @@ __device__ __forceinline__ float fmin3(float a, float b, float c)
 }
 
 // ---------------------------------------------------------------------------
-// Segment words.  A dense FP32 state vector is followed (after its NF planes)
-// by a small record per segment, 64 consecutive cells of one row: for every
-// phase one bit that is clear only where the phase is exactly +0 in all 64
-// cells, and the same for the segment's first and last cell alone (what the
+// Segment words.  A dense state vector is followed (after its NF planes) by a
+// small record per segment, 64 consecutive cells of one row (32 in FP64): for
+// every phase one bit that is clear only where the phase is exactly +0 in all
+// of them, and the same for the segment's first and last cell alone (what the
 // neighbouring segments' x differences read).  A warp of a two-cell pass owns
 // one segment: it visits only the phases that are set in a word its results
 // depend on (its own, the y/z neighbours', the facing edge cells' and those of
@@ -135,21 +135,24 @@ __device__ __forceinline__ float fmin3(float a, float b, float c)
 // phases are present nearly everywhere, and the loads of the words would only
 // lengthen each warp's chain.
 // ---------------------------------------------------------------------------
-constexpr int SEG_CELLS = 2 * VTX;
 constexpr int SEG_MIN_PHASES = 4;
 enum { SEG_ANY = 0, SEG_FIRST = 1, SEG_LAST = 2, SEG_KINDS = 3 };
 
 __host__ __device__ inline int seg_words(int N) { return (N + 31) / 32; }
 __host__ __device__ inline long long seg_count(const Geom &g)
 {
-    return (long long)((g.nx + SEG_CELLS - 1) / SEG_CELLS) * g.ny * g.nz;
+    return (long long)((g.nx + g.segc - 1) / g.segc) * g.ny * g.nz;
 }
-// Whether the state vectors of a problem carry segment words (dense FP32
-// storage; slots and masked are the storage options).
-__host__ __device__ inline bool seg_eligible(const Geom &g, bool slots, bool masked)
+// Whether the state vectors of a problem carry segment words (dense storage
+// of either precision; slots and masked are the storage options).
+__host__ __device__ inline bool seg_eligible(const Geom &g, int precision, bool slots, bool masked)
 {
-    return !slots && !masked && g.simplex == SIMPLEX_STANDARD && vec_eligible(g) && g.N > SEG_MIN_PHASES;
+    return !slots && !masked && g.simplex == SIMPLEX_STANDARD && g.N > SEG_MIN_PHASES &&
+           (precision == 64 ? seg_count(g) * SEG_KINDS * 4 < 0x7fffffffLL : vec_eligible(g));
 }
+// Cells of a segment: what a warp of the passes owns.
+__host__ __device__ constexpr int seg_length(int precision) { return precision == 64 ? 32 : 2 * VTX; }
+
 // Words of one state vector.
 __host__ __device__ inline long long seg_vec_words(const Geom &g) { return seg_count(g) * SEG_KINDS * seg_words(g.N); }
 
@@ -165,9 +168,9 @@ __device__ __forceinline__ unsigned *seg_at(const Geom &g, const T *vec, int q, 
 // words.
 __device__ __forceinline__ void seg_add_cell(const Geom &g, const float *vec, int x, int y, int z)
 {
-    const int tx = (g.nx + SEG_CELLS - 1) / SEG_CELLS;
-    const int q = (z * g.ny + y) * tx + x / SEG_CELLS;
-    const bool first = x % SEG_CELLS == 0, last = x % SEG_CELLS == SEG_CELLS - 1 || x == g.nx - 1;
+    const int tx = (g.nx + g.segc - 1) / g.segc;
+    const int q = (z * g.ny + y) * tx + x / g.segc;
+    const bool first = x % g.segc == 0, last = x % g.segc == g.segc - 1 || x == g.nx - 1;
     const long long i = ((long long)z * g.ny + y) * g.nx + x;
     for (int w = 0; w < seg_words(g.N); ++w) {
         unsigned m = 0u;
