@@ -2219,10 +2219,10 @@ int pf_create(const pf_params *p, void *cuda_stream, pf_handle **out)
     std::vector<signed char> pt(N);
     for (int a = 0; a < N; ++a) pt[a] = (signed char)h->ptype[a];
     std::vector<float> fa(h->A.begin(), h->A.end()), fb(h->B.begin(), h->B.end()), fl(h->L.begin(), h->L.end());
-    if (slots && N >= 2) {
+    if (h->prec == 32 && N >= 2) {
         // one value off the diagonal of every table (grain growth with equal
-        // gamma and M): the slot passes read it from the constants, which is
-        // the same FP32 value (same bits) the gather would return
+        // gamma and M, any two-phase problem): the FP32 passes read it from the
+        // constants, which is the same value (same bits) the gather would return
         bool same = true;
         for (int a = 0; a < N && same; ++a)
             for (int b = 0; b < N && same; ++b)

@@ -33,6 +33,25 @@ constexpr int MAXACT = 12;      // nontrivial phases per cell in the fast (share
 constexpr int WIDEACT = 64;     // ... in the per-thread fallback list of crowded cells
 constexpr int TX = 32, TY = 8;  // cells per block: 32 (x) by 8 (y), one z plane
 constexpr int BLOCK = TX * TY;
+// Cells of a warp in the masked and slot passes: a WARP_X x (32 / WARP_X) tile
+// of the block.  A compact tile holds fewer distinct phases than 32 cells in a
+// row, and the masked walk visits the union of its lanes' phases: 192^3 x 32
+// masked grains 10.47 / 9.97 / 10.4 ms, 160^3 pores with solute 28.2 / 25.5 /
+// 25.3 ms at 32 / 16 / 8 (14.3 and 35.6 against 11.7 and 27.6 ms at 4 and 16
+// before the sums moved into registers).
+#ifndef PF_WARP_X
+#define PF_WARP_X 16
+#endif
+constexpr int WARP_X = PF_WARP_X;
+
+// Position of a thread's cell in its block, warps covering tiles of W cells in x.
+template <int W>
+__device__ __forceinline__ void tile_cell(int tid, int &x, int &y)
+{
+    const int lane = tid & 31, warp = tid >> 5;
+    x = (warp % (TX / W)) * W + lane % W;
+    y = (warp / (TX / W)) * (32 / W) + lane / W;
+}
 
 // Stage combination a0 p0 + a1 v + a2 p2 of every pass, whose coefficients
 // sum to one (affine combinations of states, Eq. sts, Alg. ssp2, SSP(10)4),
@@ -76,7 +95,7 @@ struct Geom : GeomConst<double> {
     int slots;                          // 1: per-cell phase slots (FP32; see pf_slots.cuh)
     int seg, segc;                      // 1: state vectors carry segment words (see pf_vec.cuh);
                                         // cells of a segment
-    int uni;                            // slot passes: 1 if every off-diagonal entry of each
+    int uni;                            // FP32 passes: 1 if every off-diagonal entry of each
     float uA, uB, uL;                   // FP32 table A, B, L is the same value (these), which
                                         // the pairwise sums then use instead of gathers
     GeomConst<float> cf;                // the FP64 constants of the base, as float
@@ -234,9 +253,15 @@ __device__ __forceinline__ T tabs(T v) { return v < (T)0 ? -v : v; }
 #ifndef PF_DENSE_ROLLED
 #define PF_DENSE_ROLLED 0
 #endif
-// ... and of its masked-storage instantiations.
+// ... and of its masked-storage instantiations without a concentration (5: 192^3
+// x 32 grains 12.0 -> 12.6 ms, 3: 10.0 -> 10.9 ms).
 #ifndef PF_MASK_MINB
 #define PF_MASK_MINB 4
+#endif
+// With a concentration: 3 blocks at 80 registers, 4 spill 190 bytes a thread
+// (160^3 pores, 65 phases: 28.5 -> 27.2 ms).
+#ifndef PF_MASK_MINB_K1
+#define PF_MASK_MINB_K1 3
 #endif
 
 // Streaming load that does not allocate in L1 (pointwise stage inputs are
@@ -1330,6 +1355,42 @@ __device__ __forceinline__ unsigned word_bits(int N, int w)
     return r >= 32 ? 0xffffffffu : (r <= 0 ? 0u : ((1u << r) - 1u));
 }
 
+// Pairwise sums of a cell with at most R listed phases and uniform
+// coefficients (Geom::uni), in registers: t[k] = A lap_k + B phi_k is what phase
+// k adds to the derivative of every other phase, ch[k] the chemical part of its
+// own derivative, rk[k] the resulting RHS; entries k >= nz are absent (t = 0).
+// Terms and order are those of the loops over the tables: an absent term adds
+// +0 to a sum that is never -0.  Most cells list two or three phases, and the
+// loops cost a warp (largest nz)^2 iterations of two gathers and three
+// shared-memory loads each (256^3 x 32 dense grains 33.3 -> 27.9 ms, 192^3
+// masked 11.7 -> 10.0 ms, 160^3 pores with solute 27.6 -> 25.5 ms).
+constexpr int UNI_REG = 4;
+template <int KC, int R>
+__device__ __forceinline__ void uni_rhs(int nz, const float (&t)[R], const float (&ch)[R], float uL, float (&rk)[R])
+{
+    float d[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        d[k] = 0.0f;
+#pragma unroll
+        for (int k2 = 0; k2 < R; ++k2)
+            if (k2 != k) d[k] = d[k] + t[k2];
+        if (KC) d[k] = d[k] + ch[k];
+    }
+    const float inz = nz > 1 ? 1.0f / (float)nz : 0.0f;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        float s = 0.0f;
+#pragma unroll
+        for (int k2 = 0; k2 < R; ++k2) {
+            if (k2 == k) continue;
+            const float q = s + uL * (d[k] - d[k2]);
+            s = k2 < nz ? q : s;
+        }
+        rk[k] = nz > 1 ? -(s * inz) : 0.0f;
+    }
+}
+
 // Per-cell body of the FP32 fast path in masked storage (N <= 32 NW).  The
 // arithmetic and its order are those of fast_cell; what changes is which
 // phases are visited: the warp walks the union of its lanes' occupied phases
@@ -1517,42 +1578,62 @@ __device__ __forceinline__ void masked_cell(const Geom &g, const Pass<float> &P,
         for (int f = 0; f < NFACE; ++f) acc = acc + mf[f] * (num_n[f] / den_n[f] - mu);
         rc = acc * idx2;
     }
-    // variational derivative and pairwise sum over the listed phases
-    for (int k = 0; k < nz; ++k) {
-        const int a = S.id[k][tid];
-        const T *Aa = tabA + a * N, *Ba = tabB + a * N;
-        T d = (T)0;
-        for (int k2 = 0; k2 < nz; ++k2) {
-            if (k2 == k) continue;
-            const int b = S.id[k2][tid];
-            d = d + (ldg(Aa + b) * S.lap[k2][tid] + ldg(Ba + b) * S.cen[k2][tid]);
-        }
-        if (KC) {
-            const int t = ptype[a];
-            d = d + (-(mu * mu) / ((T)2 * gc.k[t]) - mu * gc.c0[t]);
-        }
-        S.dl[k][tid] = d;
+    // variational derivative and pairwise sum over the listed phases; chemical
+    // part of the derivative per type
+    T chem[2] = {(T)0, (T)0};
+    if (KC && nz > 0) {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) chem[t] = -(mu * mu) / ((T)2 * gc.k[t]) - mu * gc.c0[t];
     }
-    const T inz = nz > 1 ? (T)1 / (T)nz : (T)0;
-    for (int k = 0; k < nz; ++k) {
-        T rk = (T)0;
-        if (nz > 1) {
+    if (g.uni && nz <= UNI_REG) {
+        if (nz > 0) {
+            T t[UNI_REG], ch[UNI_REG], rk[UNI_REG];
+#pragma unroll
+            for (int k = 0; k < UNI_REG; ++k) {
+                t[k] = k < nz ? g.uA * S.lap[k][tid] + g.uB * S.cen[k][tid] : (T)0;
+                ch[k] = KC && k < nz ? (ptype[S.id[k][tid]] ? chem[1] : chem[0]) : (T)0;
+            }
+            uni_rhs<KC, UNI_REG>(nz, t, ch, g.uL, rk);
+#pragma unroll
+            for (int k = 0; k < UNI_REG; ++k)
+                if (k < nz) S.lap[k][tid] = rk[k];      // the list now holds the RHS
+        }
+    } else {
+        for (int k = 0; k < nz; ++k) {
             const int a = S.id[k][tid];
-            const T *La = tabL + a * N;
-            const T dk = S.dl[k][tid];
-            T s = (T)0;
+            const T *Aa = tabA + a * N, *Ba = tabB + a * N;
+            T d = (T)0;
             for (int k2 = 0; k2 < nz; ++k2) {
                 if (k2 == k) continue;
-                s = s + ldg(La + S.id[k2][tid]) * (dk - S.dl[k2][tid]);
+                const int b = S.id[k2][tid];
+                d = d + (ldg(Aa + b) * S.lap[k2][tid] + ldg(Ba + b) * S.cen[k2][tid]);
             }
-            rk = -(s * inz);
+            if (KC) d = d + (ptype[a] ? chem[1] : chem[0]);
+            S.dl[k][tid] = d;
         }
-        S.lap[k][tid] = rk;                 // the list now holds the RHS
-        if (ERR) {
+        const T inz = nz > 1 ? (T)1 / (T)nz : (T)0;
+        for (int k = 0; k < nz; ++k) {
+            T rk = (T)0;
+            if (nz > 1) {
+                const int a = S.id[k][tid];
+                const T *La = tabL + a * N;
+                const T dk = S.dl[k][tid];
+                T s = (T)0;
+                for (int k2 = 0; k2 < nz; ++k2) {
+                    if (k2 == k) continue;
+                    s = s + ldg(La + S.id[k2][tid]) * (dk - S.dl[k2][tid]);
+                }
+                rk = -(s * inz);
+            }
+            S.lap[k][tid] = rk;
+        }
+    }
+    if (ERR) {
+        for (int k = 0; k < nz; ++k) {
             const int a = S.id[k][tid];
             const long long fo = (long long)a * Vs;
             const T p0v = ldg(P.p0 + fo + i), v0 = S.cen[k][tid], r0v = ldg(P.r0in + fo + i);
-            const T sr = r0v + rk;
+            const T sr = r0v + S.lap[k][tid];
             T e = ((T)12 * (p0v - v0) + ((T)6 * dt) * sr) * ((T)1 / (T)15);
             const T trial = p0v + (dt * (T)0.5) * sr;
             if (trial < (T)0 || trial > (T)1) e = (T)0;
@@ -2008,8 +2089,10 @@ __device__ __forceinline__ void fast_body(const Geom &g, const Pass<float> &P, c
     ListSmem<float> &S = *reinterpret_cast<ListSmem<float> *>(smem_raw);
     const int tid = threadIdx.x;
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    const int x = blockIdx.x * TX + (tid % TX);
-    const int y = blockIdx.y * TY + (tid / TX);
+    int tx, ty;
+    tile_cell<MASK ? WARP_X : TX>(tid, tx, ty);
+    const int x = blockIdx.x * TX + tx;
+    const int y = blockIdx.y * TY + ty;
     const int z = blockIdx.z;
     double esum = 0.0;
     long long ecnt = 0;
@@ -2055,7 +2138,7 @@ __device__ __forceinline__ void fast_body(const Geom &g, const Pass<float> &P, c
 }
 
 template <int DIM, int KC, unsigned SIG, int NMAX, bool MASK = false>
-__global__ void __launch_bounds__(BLOCK, MASK ? PF_MASK_MINB : PF_FAST_MINB)
+__global__ void __launch_bounds__(BLOCK, MASK ? (KC ? PF_MASK_MINB_K1 : PF_MASK_MINB) : PF_FAST_MINB)
 fast_kernel(const __grid_constant__ Geom g, const __grid_constant__ Pass<float> P, const float *__restrict__ tabA,
             const float *__restrict__ tabB, const float *__restrict__ tabL, const signed char *__restrict__ ptype)
 {

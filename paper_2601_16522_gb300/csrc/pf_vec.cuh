@@ -47,8 +47,10 @@ constexpr int VCELLS = 2 * VBLOCK;   // 256 cells per block
 #define PF_VEC_ACT_LIGHT 6
 #endif
 // Resident blocks per SM the register budget targets.
+// (RKL2 body: 6 blocks at 80 registers; 256^3 x 32 grains, three attempts 24.0
+// -> 22.7 ms against 5 at 96.)
 #ifndef PF_VEC_MINB
-#define PF_VEC_MINB 5
+#define PF_VEC_MINB 6
 #endif
 #ifndef PF_VEC_MINB_LIGHT
 #define PF_VEC_MINB_LIGHT 7
@@ -236,7 +238,9 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
         C[c].nz = 0; C[c].bestid = -1; C[c].nc = 0; C[c].best = (T)-1; C[c].ssum = (T)0;
         C[c].changed = false; C[c].nzcnt = 0; C[c].es = 0.0; C[c].ec = 0;
     }
-    bool crowd[2] = {false, false};
+    unsigned crowd = 0u;       // bit c: cell c goes to the wide pass
+    double es = 0.0;           // error partials of the cells (MODE_ERR)
+    long long ec = 0;
     if (y < g.ny) {   // warp-uniform (a warp is one row)
         const bool here = x < g.nx;
         const int row = z * g.ny + y;
@@ -464,8 +468,9 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                 visited[ty][w] = U;
                 if (R0OUT) fixed[ty][w] = 0u;
             }
-            // two phases per iteration: the loads of the next phase are in flight
-            // while the current one is processed, without register copies
+            // the loads of the next phase are in flight while the current one is
+            // processed (one copy of the code: a second one instead of the
+            // register copies costs 0.2 ms of 24 in instruction fetches)
             unsigned m = U;
             if (m) {
                 VPhase qa, qb;
@@ -482,14 +487,9 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
                     }
                     process(w, a, pa, qa);
                     if (b < 0) break;
-                    a = __ffs(m) - 1;
-                    if (a >= 0) {
-                        m &= m - 1u;
-                        pa = (long long)(32 * w + a) * Vs;
-                        fetch(a, pa, qa);
-                    }
-                    process(w, b, pb, qb);
-                    if (a < 0) break;
+                    a = b;
+                    pa = pb;
+                    qa = qb;
                 }
             }
         }
@@ -560,188 +560,220 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
             }
         }
 
-        // ---- pairwise sums over each cell's list ----------------------------
-#pragma unroll
+        // ---- the two cells in turn, in one copy of the code: with a copy for
+        // each the kernel outgrew the instruction cache (1.9 of 11 stall cycles
+        // an instruction; 256^3 x 32 grains, three attempts: 27.8 -> 24.0 ms) ---
+#pragma unroll 1
         for (int c = 0; c < 2; ++c) {
-            VCell &Cc = C[c];
+            VCell Cc = c == 0 ? C[0] : C[1];
+            const T muc = c == 0 ? mu[0] : mu[1], rcc = c == 0 ? rc[0] : rc[1], ccc = c == 0 ? cc[0] : cc[1];
             const int slot = c * VBLOCK + tid;
-            if (!here) continue;
-            if (Cc.nz > VACT) { crowd[c] = true; continue; }
-            const int nz = Cc.nz;
-            for (int k = 0; k < nz; ++k) {
-                const int a = S.id[k][slot];
-                const T *Aa = tabA + a * N, *Ba = tabB + a * N;
-                T d = (T)0;
-                for (int k2 = 0; k2 < nz; ++k2) {
-                    if (k2 == k) continue;
-                    const int b = S.id[k2][slot];
-                    d = d + (__ldg(Aa + b) * S.lap[k2][slot] + __ldg(Ba + b) * S.cen[k2][slot]);
+            const bool full = Cc.nz > VACT;      // crowded: left to the wide pass
+            // pairwise sums over the cell's list
+            auto pairs = [&]() {
+                if (!here || full) return;
+                const int nz = Cc.nz;
+                // chemical part of the derivative per type
+                T chem[2] = {(T)0, (T)0};
+                if (KC && nz > 0) {
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) chem[t] = -(muc * muc) / ((T)2 * gc.k[t]) - muc * gc.c0[t];
                 }
-                if (KC) {
-                    const int t = ptype[a];
-                    d = d + (-(mu[c] * mu[c]) / ((T)2 * gc.k[t]) - mu[c] * gc.c0[t]);
-                }
-                S.dl[k][slot] = d;
-            }
-            const T inz = nz > 1 ? (T)1 / (T)nz : (T)0;
-            for (int k = 0; k < nz; ++k) {
-                T rk = (T)0;
-                const int a = S.id[k][slot];
-                if (nz > 1) {
-                    const T *La = tabL + a * N;
-                    const T dk = S.dl[k][slot];
-                    T s = (T)0;
-                    for (int k2 = 0; k2 < nz; ++k2) {
-                        if (k2 == k) continue;
-                        s = s + __ldg(La + S.id[k2][slot]) * (dk - S.dl[k2][slot]);
-                    }
-                    rk = -(s * inz);
-                }
-                S.lap[k][slot] = rk;              // the list now holds the RHS
-                const long long fo = (long long)a * Vs + i + c;
-                if (ERR) {
-                    const T p0v = __ldg(P.p0 + fo), v0 = S.cen[k][slot], r0v = __ldg(P.r0in + fo);
-                    const T sr = r0v + rk;
-                    T e = ((T)12 * (p0v - v0) + ((T)6 * dt) * sr) * ((T)1 / (T)15);
-                    const T trial = p0v + (dt * (T)0.5) * sr;
-                    if (trial < (T)0 || trial > (T)1) e = (T)0;
-                    if (e != (T)0) {
-                        const T w = rph * fmaxf(fabsf(p0v), fabsf(v0)) + aph;
-                        const T q = e / w;
-                        Cc.es += (double)(q * q);
-                        Cc.nc++;
-                    }
-                    if (R0OUT) P.r0out[fo] = rk;   // F(u^{n+1}) kept for reuse
-                } else {
-                    T acc = S.val[k][slot] + b1c * rk;
-                    if (PROJ) {
-                        if (acc < (T)0) { acc = (T)0; Cc.changed = true; }
-                        if (acc >= (T)1 && (acc > Cc.best || (acc == Cc.best && a < Cc.bestid))) {
-                            Cc.best = acc;
-                            Cc.bestid = a;
-                        }
-                        Cc.ssum = Cc.ssum + acc;
-                    }
-                    S.val[k][slot] = acc;
-                }
-            }
-        }
-
-        // ---- projection, final values, concentration ------------------------
-        auto finish = [&](int c) {
-            VCell &Cc = C[c];
-            const int slot = c * VBLOCK + tid;
-            if (!here || crowd[c]) return;
-            const int nz = Cc.nz;
-            if (ERR) {
-                Cc.ec += (Cc.nc > 0 ? Cc.nc : 2);
-                if (KC) {
-                    const long long o = (long long)N * Vs + i + c;
-                    const T un = __ldg(P.p0 + o), un1 = cc[c], rn = __ldg(P.r0in + o);
-                    const T e = ((T)12 * (un - un1) + ((T)6 * dt) * (rn + rc[c])) * ((T)1 / (T)15);
-                    const T w = P.c.r_c * fmaxf(fabsf(un + gc.cref), fabsf(un1 + gc.cref)) + P.c.a_c;
-                    const T q = e / w;
-                    Cc.es += (double)(q * q);
-                    Cc.ec += 1;
-                    if (R0OUT) P.r0out[o] = rc[c];
-                }
-                return;
-            }
-            bool rewrite = false;     // inactive nonzero entries need their final value
-            if (PROJ) {
-                if (Cc.bestid >= 0) {
-                    // the winner becomes 1, the others 0: a change unless the
-                    // winner is exactly 1 and every other phase already zero.
-                    // Unlisted entries need rewriting only where nonzero
-                    // (nzcnt of them, the winner among them if unlisted).
-                    bool listed = false, others = false;
-                    for (int k = 0; k < nz; ++k) {
-                        if (S.id[k][slot] == Cc.bestid) listed = true;
-                        else if (S.val[k][slot] != (T)0) others = true;
-                    }
-                    const int unl_others = Cc.nzcnt - (listed ? 0 : 1);
-                    if (others || unl_others > 0 || Cc.best != (T)1) Cc.changed = true;
-                    rewrite = unl_others > 0 || (!listed && Cc.best != (T)1);
-                    Cc.ssum = (T)1;
-                }
-                if (!(Cc.ssum > (T)0)) raise_flag(P.flag, FLAG_SIMPLEX);
-            }
-            const T inv = (Cc.ssum > (T)0) ? (T)1 / Cc.ssum : (T)1;
-            if (PROJ && Cc.bestid < 0 && inv != (T)1 && Cc.nzcnt > 0) rewrite = true;
-            const bool fix = R0OUT && P.fix_first && Cc.changed;
-            // listed phases
-            for (int k = 0; k < nz; ++k) {
-                const int a = S.id[k][slot];
-                const long long fo = (long long)a * Vs + i + c;
-                T w = S.val[k][slot];
-                if (PROJ) w = (Cc.bestid >= 0) ? ((a == Cc.bestid) ? (T)1 : (T)0) : w * inv;
-                P.out[fo] = w;
-                S.val[k][slot] = w;
-                if (R0OUT) {
-                    T r = S.lap[k][slot];
-                    if (fix) r = (w - S.cen[k][slot]) * ib1;
-                    P.r0out[fo] = r;
-                }
-            }
-            // phases not listed whose written value is nonzero (rare outside
-            // bulk cells): the >= 1 rule or the normalisation
-            if (rewrite) {
-                int kk = 0;
-                for (int wd = 0; wd < nw; ++wd)
-                    for (unsigned m = visited[ty][wd]; m; m &= m - 1u) {
-                        const int a = 32 * wd + __ffs(m) - 1;
-                        if (kk < nz && S.id[kk][slot] == a) { kk++; continue; }
+                // the RHS rk of listed phase k: error term, or stage value, clamp,
+                // >= 1 candidate and sum
+                auto listed = [&](int k, T rk) {
+                    const int a = S.id[k][slot];
+                    if (R0OUT) S.lap[k][slot] = rk;       // the list now holds the RHS
+                    if (ERR) {
                         const long long fo = (long long)a * Vs + i + c;
-                        const T o = P.out[fo];
-                        if (o == (T)0) continue;
-                        const T w = (Cc.bestid >= 0) ? ((a == Cc.bestid) ? (T)1 : (T)0) : o * inv;
-                        P.out[fo] = w;
-                        if (fix) {
-                            P.r0out[fo] = (w - __ldg(P.in + fo)) * ib1;
-                            if (seg) atomicOr(&fixed[ty][wd], 1u << (a & 31));
+                        const T p0v = __ldg(P.p0 + fo), v0 = S.cen[k][slot], r0v = __ldg(P.r0in + fo);
+                        const T sr = r0v + rk;
+                        T e = ((T)12 * (p0v - v0) + ((T)6 * dt) * sr) * ((T)1 / (T)15);
+                        const T trial = p0v + (dt * (T)0.5) * sr;
+                        if (trial < (T)0 || trial > (T)1) e = (T)0;
+                        if (e != (T)0) {
+                            const T w = rph * fmaxf(fabsf(p0v), fabsf(v0)) + aph;
+                            const T q = e / w;
+                            Cc.es += (double)(q * q);
+                            Cc.nc++;
                         }
+                        if (R0OUT) P.r0out[fo] = rk;   // F(u^{n+1}) kept for reuse
+                    } else {
+                        T acc = S.val[k][slot] + b1c * rk;
+                        if (PROJ) {
+                            if (acc < (T)0) { acc = (T)0; Cc.changed = true; }
+                            if (acc >= (T)1 && (acc > Cc.best || (acc == Cc.best && a < Cc.bestid))) {
+                                Cc.best = acc;
+                                Cc.bestid = a;
+                            }
+                            Cc.ssum = Cc.ssum + acc;
+                        }
+                        S.val[k][slot] = acc;
                     }
-            }
-            if (KC) {
-                const long long o = (long long)N * Vs + i + c;
-                // the small increments are summed first: c is rounded once per stage
-                T d = b1c * rc[c];
-                if (HR0) d = d + b0c * __ldg(P.r0in + o);
-                if (HP0) d = d + a0c * (__ldg(P.p0 + o) - cc[c]);
-                if (HP2) d = d + a2c * (__ldg(P.p2 + o) - cc[c]);
-                const T acc = cc[c] + d;
-                if (!isfinite(acc)) raise_flag(P.flag, FLAG_NONFINITE);
-                if (R0OUT) P.r0out[o] = rc[c];
-                P.out[o] = acc;
-            }
-        };
+                };
+                if (g.uni && nz <= UNI_REG) {
+                    if (nz == 0) return;
+                    T t[UNI_REG], ch[UNI_REG], rk[UNI_REG];
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            finish(c);
-            if (ERR ? !R0OUT : false) continue;
-            if (!seg) continue;
-            // the listed phases' part of the output words
-            const int slot = c * VBLOCK + tid;
-            const int nz = here && !crowd[c] ? C[c].nz : 0;
-            for (int w = 0; w < nw; ++w) {
-                unsigned mv = 0u, ml = 0u;
+                    for (int k = 0; k < UNI_REG; ++k) {
+                        t[k] = k < nz ? g.uA * S.lap[k][slot] + g.uB * S.cen[k][slot] : (T)0;
+                        ch[k] = KC && k < nz ? (ptype[S.id[k][slot]] ? chem[1] : chem[0]) : (T)0;
+                    }
+                    uni_rhs<KC, UNI_REG>(nz, t, ch, g.uL, rk);
+#pragma unroll
+                    for (int k = 0; k < UNI_REG; ++k)
+                        if (k < nz) listed(k, rk[k]);
+                    return;
+                }
                 for (int k = 0; k < nz; ++k) {
                     const int a = S.id[k][slot];
-                    if (nw > 1 && (a >> 5) != w) continue;
-                    ml |= 1u << (a & 31);
-                    if (!ERR && __float_as_uint(S.val[k][slot]) != 0u) mv |= 1u << (a & 31);
+                    const T *Aa = tabA + a * N, *Ba = tabB + a * N;
+                    T d = (T)0;
+                    for (int k2 = 0; k2 < nz; ++k2) {
+                        if (k2 == k) continue;
+                        const int b = S.id[k2][slot];
+                        d = d + (__ldg(Aa + b) * S.lap[k2][slot] + __ldg(Ba + b) * S.cen[k2][slot]);
+                    }
+                    if (KC) d = d + (ptype[a] ? chem[1] : chem[0]);
+                    S.dl[k][slot] = d;
                 }
-                if (!ERR) {
-                    const unsigned r = __reduce_or_sync(ALL, mv), e = __shfl_sync(ALL, mv, c == 0 ? 0 : lastlane);
-                    if (lane == w) {
-                        w_any |= r;
-                        if (c == 0) w_first |= e;
-                        else w_last |= e;
+                const T inz = nz > 1 ? (T)1 / (T)nz : (T)0;
+                for (int k = 0; k < nz; ++k) {
+                    T rk = (T)0;
+                    if (nz > 1) {
+                        const T *La = tabL + S.id[k][slot] * N;
+                        const T dk = S.dl[k][slot];
+                        T s = (T)0;
+                        for (int k2 = 0; k2 < nz; ++k2) {
+                            if (k2 == k) continue;
+                            s = s + __ldg(La + S.id[k2][slot]) * (dk - S.dl[k2][slot]);
+                        }
+                        rk = -(s * inz);
+                    }
+                    listed(k, rk);
+                }
+            };
+            pairs();
+            __syncwarp();     // the lanes meet again after sums of different lengths
+
+            // projection, final values, concentration
+            // word of the cell's listed phases, and of those with a value that is
+            // not +0 (problems of one word)
+            unsigned lml = 0u, lmv = 0u;
+            auto finish = [&]() {
+                if (!here || full) return;
+                const int nz = Cc.nz;
+                if (ERR) {
+                    Cc.ec += (Cc.nc > 0 ? Cc.nc : 2);
+                    if (KC) {
+                        const long long o = (long long)N * Vs + i + c;
+                        const T un = __ldg(P.p0 + o), un1 = ccc, rn = __ldg(P.r0in + o);
+                        const T e = ((T)12 * (un - un1) + ((T)6 * dt) * (rn + rcc)) * ((T)1 / (T)15);
+                        const T w = P.c.r_c * fmaxf(fabsf(un + gc.cref), fabsf(un1 + gc.cref)) + P.c.a_c;
+                        const T q = e / w;
+                        Cc.es += (double)(q * q);
+                        Cc.ec += 1;
+                        if (R0OUT) P.r0out[o] = rcc;
+                    }
+                    return;
+                }
+                bool rewrite = false;     // inactive nonzero entries need their final value
+                if (PROJ) {
+                    if (Cc.bestid >= 0) {
+                        // the winner becomes 1, the others 0: a change unless the
+                        // winner is exactly 1 and every other phase already zero.
+                        // Unlisted entries need rewriting only where nonzero
+                        // (nzcnt of them, the winner among them if unlisted).
+                        bool listed = false, others = false;
+                        for (int k = 0; k < nz; ++k) {
+                            if (S.id[k][slot] == Cc.bestid) listed = true;
+                            else if (S.val[k][slot] != (T)0) others = true;
+                        }
+                        const int unl_others = Cc.nzcnt - (listed ? 0 : 1);
+                        if (others || unl_others > 0 || Cc.best != (T)1) Cc.changed = true;
+                        rewrite = unl_others > 0 || (!listed && Cc.best != (T)1);
+                        Cc.ssum = (T)1;
+                    }
+                    if (!(Cc.ssum > (T)0)) raise_flag(P.flag, FLAG_SIMPLEX);
+                }
+                const T inv = (Cc.ssum > (T)0) ? (T)1 / Cc.ssum : (T)1;
+                if (PROJ && Cc.bestid < 0 && inv != (T)1 && Cc.nzcnt > 0) rewrite = true;
+                const bool fix = R0OUT && P.fix_first && Cc.changed;
+                // listed phases
+                for (int k = 0; k < nz; ++k) {
+                    const int a = S.id[k][slot];
+                    const long long fo = (long long)a * Vs + i + c;
+                    T w = S.val[k][slot];
+                    if (PROJ) w = (Cc.bestid >= 0) ? ((a == Cc.bestid) ? (T)1 : (T)0) : w * inv;
+                    P.out[fo] = w;
+                    if (nw > 1) S.val[k][slot] = w;
+                    lml |= 1u << (a & 31);
+                    if (__float_as_uint(w) != 0u) lmv |= 1u << (a & 31);
+                    if (R0OUT) {
+                        T r = S.lap[k][slot];
+                        if (fix) r = (w - S.cen[k][slot]) * ib1;
+                        P.r0out[fo] = r;
                     }
                 }
-                if (R0OUT) {
-                    const unsigned r = __reduce_or_sync(ALL, ml);
-                    if (lane == w) w_r0 |= r;
+                // phases not listed whose written value is nonzero (rare outside
+                // bulk cells): the >= 1 rule or the normalisation
+                if (rewrite) {
+                    int kk = 0;
+                    for (int wd = 0; wd < nw; ++wd)
+                        for (unsigned m = visited[ty][wd]; m; m &= m - 1u) {
+                            const int a = 32 * wd + __ffs(m) - 1;
+                            if (kk < nz && S.id[kk][slot] == a) { kk++; continue; }
+                            const long long fo = (long long)a * Vs + i + c;
+                            const T o = P.out[fo];
+                            if (o == (T)0) continue;
+                            const T w = (Cc.bestid >= 0) ? ((a == Cc.bestid) ? (T)1 : (T)0) : o * inv;
+                            P.out[fo] = w;
+                            if (fix) {
+                                P.r0out[fo] = (w - __ldg(P.in + fo)) * ib1;
+                                if (seg) atomicOr(&fixed[ty][wd], 1u << (a & 31));
+                            }
+                        }
+                }
+                if (KC) {
+                    const long long o = (long long)N * Vs + i + c;
+                    // the small increments are summed first: c is rounded once per stage
+                    T d = b1c * rcc;
+                    if (HR0) d = d + b0c * __ldg(P.r0in + o);
+                    if (HP0) d = d + a0c * (__ldg(P.p0 + o) - ccc);
+                    if (HP2) d = d + a2c * (__ldg(P.p2 + o) - ccc);
+                    const T acc = ccc + d;
+                    if (!isfinite(acc)) raise_flag(P.flag, FLAG_NONFINITE);
+                    if (R0OUT) P.r0out[o] = rcc;
+                    P.out[o] = acc;
+                }
+            };
+            finish();
+            if (here && full) crowd |= 1u << c;
+            if (ERR) { es += Cc.es; ec += Cc.ec; }
+            if (seg && (!ERR || R0OUT)) {
+                // the listed phases' part of the output words
+                const int nz = here && !full ? Cc.nz : 0;
+                for (int w = 0; w < nw; ++w) {
+                    unsigned mv = lmv, ml = lml;
+                    if (nw > 1) mv = ml = 0u;
+                    for (int k = 0; (nw > 1 || ERR) && k < nz; ++k) {
+                        const int a = S.id[k][slot];
+                        if (nw > 1 && (a >> 5) != w) continue;
+                        ml |= 1u << (a & 31);
+                        if (!ERR && __float_as_uint(S.val[k][slot]) != 0u) mv |= 1u << (a & 31);
+                    }
+                    if (!ERR) {
+                        const unsigned r = __reduce_or_sync(ALL, mv), e = __shfl_sync(ALL, mv, c == 0 ? 0 : lastlane);
+                        if (lane == w) {
+                            w_any |= r;
+                            if (c == 0) w_first |= e;
+                            else w_last |= e;
+                        }
+                    }
+                    if (R0OUT) {
+                        const unsigned r = __reduce_or_sync(ALL, ml);
+                        if (lane == w) w_r0 |= r;
+                    }
                 }
             }
         }
@@ -764,10 +796,10 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
     // from there.  The block appends one entry: its index and a 256-bit mask.
     __shared__ unsigned cmask[VCELLS / 32];
     if (tid < VCELLS / 32) cmask[tid] = 0u;
-    if (__syncthreads_or(crowd[0] || crowd[1])) {
+    if (__syncthreads_or(crowd != 0u)) {
 #pragma unroll
         for (int c = 0; c < 2; ++c)
-            if (crowd[c]) {
+            if ((crowd >> c) & 1u) {
                 const int bit = ty * (2 * VTX) + 2 * lane + c;
                 atomicOr(&cmask[bit >> 5], 1u << (bit & 31));
             }
@@ -780,7 +812,7 @@ __device__ __forceinline__ void vec_body(const Geom &g, const Pass<float> &P, co
             for (int w = 0; w < VCELLS / 32; ++w) ent[1 + w] = (int)cmask[w];
         }
     }
-    if (ERR) block_partials(C[0].es + C[1].es, C[0].ec + C[1].ec, P.part_sum, P.part_cnt, bid, P.part_n, nblk);
+    if (ERR) block_partials(es, ec, P.part_sum, P.part_cnt, bid, P.part_n, nblk);
     // the step is counted by the wide pass, after the crowded cells, where
     // there can be any
     if (P.count_step && !vec_crowds(g)) count_step_done(P.flag, nblk);
