@@ -226,7 +226,8 @@ def sunit(kc, fname):
     for d in (2, 3):
         for sg in SIGS + ["SIG_RHS"]:
             L.append("    if (g.dim == %d && sig == (%s)) {" % (d, sg))
-            L.append("        slot_kernel<%d, %d, %s><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);" % (d, kc, sg))
+            L.append("        if (g.uni) slot_kernel<%d, %d, %s, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);" % (d, kc, sg))
+            L.append("        else slot_kernel<%d, %d, %s, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);" % (d, kc, sg))
             L.append("        return (int)cudaGetLastError();")
             L.append("    }")
     L.append("    *done = false;")

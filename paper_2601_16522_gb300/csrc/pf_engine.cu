@@ -135,23 +135,18 @@ __global__ void unpack_kernel(const T *__restrict__ src, double *__restrict__ ph
 __global__ void slot_pack_dense(const double *__restrict__ phi, const double *__restrict__ c, float *__restrict__ dst,
                                 long long V, int Vs, int N, int K, double cref, int *flag)
 {
-    unsigned short *ids = reinterpret_cast<unsigned short *>(dst + (long long)pfk::NSLOT * Vs);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x) {
         int cnt = 0;
+        pfk::SlotWriter W;
+        W.start();
         for (int a = 0; a < N; ++a) {
             const float v = (float)phi[(long long)a * V + i];
             if (v == 0.0f) continue;
-            if (cnt < pfk::NSLOT) {
-                dst[(long long)cnt * Vs + i] = v;
-                ids[(long long)cnt * Vs + i] = (unsigned short)a;
-            }
+            if (cnt < pfk::NSLOT) W.push(v, (unsigned)a, dst, Vs, (int)i);
             cnt++;
         }
         if (cnt > pfk::NSLOT) atomicOr(flag, pfk::FLAG_NZ_OVERFLOW);
-        for (int k = cnt; k < pfk::NSLOT; ++k) {
-            dst[(long long)k * Vs + i] = 0.0f;
-            ids[(long long)k * Vs + i] = (unsigned short)pfk::SLOT_EMPTY;
-        }
+        W.finish(dst, Vs, (int)i);
         if (K) dst[(long long)pfk::SLOT_C_PLANES * Vs + i] = (float)(c[i] - cref);
     }
 }
@@ -164,7 +159,6 @@ __global__ void slot_pack_slots(const double *__restrict__ vals, const int *__re
                                 const double *__restrict__ c, float *__restrict__ dst, long long V, int Vs, int N,
                                 int K, double cref, int *flag)
 {
-    unsigned short *ids = reinterpret_cast<unsigned short *>(dst + (long long)pfk::NSLOT * Vs);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x) {
         float sv[pfk::NSLOT];
         int sid[pfk::NSLOT];
@@ -185,10 +179,10 @@ __global__ void slot_pack_slots(const double *__restrict__ vals, const int *__re
             cnt++;
         }
         if (bad) { atomicOr(flag, pfk::FLAG_NZ_OVERFLOW); cnt = 0; }
-        for (int k = 0; k < pfk::NSLOT; ++k) {
-            dst[(long long)k * Vs + i] = k < cnt ? sv[k] : 0.0f;
-            ids[(long long)k * Vs + i] = (unsigned short)(k < cnt ? sid[k] : (int)pfk::SLOT_EMPTY);
-        }
+        pfk::SlotWriter W;
+        W.start();
+        for (int k = 0; k < cnt; ++k) W.push(sv[k], (unsigned)sid[k], dst, Vs, (int)i);
+        W.finish(dst, Vs, (int)i);
         if (K) dst[(long long)pfk::SLOT_C_PLANES * Vs + i] = (float)(c[i] - cref);
     }
 }
@@ -197,13 +191,14 @@ __global__ void slot_pack_slots(const double *__restrict__ vals, const int *__re
 __global__ void slot_unpack_dense(const float *__restrict__ src, double *__restrict__ phi, double *__restrict__ c,
                                   long long V, int Vs, int N, int K, double cref)
 {
-    const unsigned short *ids = reinterpret_cast<const unsigned short *>(src + (long long)pfk::NSLOT * Vs);
+    const unsigned short *ids = pfk::slot_ids(src, Vs);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x) {
         for (int a = 0; a < N; ++a) phi[(long long)a * V + i] = 0.0;
         for (int k = 0; k < pfk::NSLOT; ++k) {
-            const unsigned a = ids[(long long)k * Vs + i];
+            const int at = pfk::slot_at(k, Vs, (int)i);
+            const unsigned a = ids[at ^ 1];
             if (a >= (unsigned)N) break;
-            phi[(long long)a * V + i] = (double)src[(long long)k * Vs + i];
+            phi[(long long)a * V + i] = (double)src[at];
         }
         if (K && c) c[i] = (double)src[(long long)pfk::SLOT_C_PLANES * Vs + i] + cref;
     }
@@ -213,12 +208,13 @@ __global__ void slot_unpack_dense(const float *__restrict__ src, double *__restr
 __global__ void slot_unpack_slots(const float *__restrict__ src, double *__restrict__ vals, int *__restrict__ idout,
                                   double *__restrict__ c, long long V, int Vs, int N, int K, double cref)
 {
-    const unsigned short *ids = reinterpret_cast<const unsigned short *>(src + (long long)pfk::NSLOT * Vs);
+    const unsigned short *ids = pfk::slot_ids(src, Vs);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x) {
         for (int k = 0; k < pfk::NSLOT; ++k) {
-            const unsigned a = ids[(long long)k * Vs + i];
+            const int at = pfk::slot_at(k, Vs, (int)i);
+            const unsigned a = ids[at ^ 1];
             const bool used = a < (unsigned)N;
-            vals[(long long)k * V + i] = used ? (double)src[(long long)k * Vs + i] : 0.0;
+            vals[(long long)k * V + i] = used ? (double)src[at] : 0.0;
             idout[(long long)k * V + i] = used ? (int)a : -1;
         }
         if (K && c) c[i] = (double)src[(long long)pfk::SLOT_C_PLANES * Vs + i] + cref;
@@ -231,12 +227,13 @@ __global__ void slot_unpack_slots(const float *__restrict__ src, double *__restr
 __global__ void slot_phase_totals(const float *__restrict__ src, long long V, int Vs, int N, double *vol,
                                   unsigned long long *mx)
 {
-    const unsigned short *ids = reinterpret_cast<const unsigned short *>(src + (long long)pfk::NSLOT * Vs);
+    const unsigned short *ids = pfk::slot_ids(src, Vs);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x)
         for (int k = 0; k < pfk::NSLOT; ++k) {
-            const unsigned a = ids[(long long)k * Vs + i];
+            const int at = pfk::slot_at(k, Vs, (int)i);
+            const unsigned a = ids[at ^ 1];
             if (a >= (unsigned)N) break;
-            const double v = (double)src[(long long)k * Vs + i];
+            const double v = (double)src[at];
             atomicAdd(vol + a, v);
             if (v > 0.0) atomicMax(mx + a, (unsigned long long)__double_as_longlong(v));
         }
