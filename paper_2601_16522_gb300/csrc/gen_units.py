@@ -46,8 +46,13 @@ def dbl_launch(kernel, arg, prep):
         for k in (0, 1):
             for r in (2, 8):
                 L.append("        if (g.dim == %d && g.K == %d && rows == %d) {" % (d, k, r))
-                L.append("            %s<%d, %d, %d><<<dgrid, DBL_TX * %d, sizeof(DblSmem<%d>), st>>>(g, %s, A, B, L, ptype);"
-                         % (kernel, d, k, r, r, r, arg))
+                inst = "%s<%d, %d, %d>" % (kernel, d, k, r)
+                shape = "dgrid, DBL_TX * %d, sizeof(DblSmem<%d>), st" % (r, r)
+                args = "g, %s, A, B, L, ptype" % arg
+                if kernel.endswith("_d"):
+                    L.append("            %s<<<%s>>>(%s);" % (inst, shape, args))
+                else:
+                    L.append("            launch_pass(%s, %s, %s);" % (inst, shape, args))
                 L.append("            return (int)cudaGetLastError();")
                 L.append("        }")
                 prep.append("    if (cudaFuncSetAttribute(%s<%d, %d, %d>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DblSmem<%d>)) != cudaSuccess) return -1;"
@@ -77,7 +82,7 @@ def unit(T, kcs, fast, fname):
         for d in (2, 3):
             for sg in SSP_SIGS:
                 L.append("        if (g.dim == %d && sig == (%s)) {" % (d, sg))
-                L.append("            fast_kernel<%d, %d, %s, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);" % (d, kc, sg))
+                L.append("            launch_pass(fast_kernel<%d, %d, %s, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);" % (d, kc, sg))
                 L.append("            return (int)cudaGetLastError();")
                 L.append("        }")
                 prep.append("    if (cudaFuncSetAttribute(fast_kernel<%d, %d, %s, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf) != cudaSuccess) return -1;" % (d, kc, sg))
@@ -105,7 +110,7 @@ def unit(T, kcs, fast, fname):
             for d in (2, 3):
                 for sg in FAST_SIGS + SSP_SIGS:
                     L.append("            if (g.dim == %d && sig == (%s)) {" % (d, sg))
-                    L.append("                fast_kernel<%d, %d, %s, %d><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);" % (d, kc, sg, nmax))
+                    L.append("                launch_pass(fast_kernel<%d, %d, %s, %d>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);" % (d, kc, sg, nmax))
                     L.append("                return (int)cudaGetLastError();")
                     L.append("            }")
                     prep.append("    if (cudaFuncSetAttribute(fast_kernel<%d, %d, %s, %d>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf) != cudaSuccess) return -1;" % (d, kc, sg, nmax))
@@ -193,7 +198,7 @@ def munit(kc, fname):
         for d in (2, 3):
             for sg in SIGS + SSP_SIGS:
                 L.append("            if (g.dim == %d && sig == (%s)) {" % (d, sg))
-                L.append("                fast_kernel<%d, %d, %s, %d, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);" % (d, kc, sg, nmax))
+                L.append("                launch_pass(fast_kernel<%d, %d, %s, %d, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);" % (d, kc, sg, nmax))
                 L.append("                return (int)cudaGetLastError();")
                 L.append("            }")
                 prep.append("    if (cudaFuncSetAttribute(fast_kernel<%d, %d, %s, %d, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smf) != cudaSuccess) return -1;" % (d, kc, sg, nmax))
@@ -226,8 +231,8 @@ def sunit(kc, fname):
     for d in (2, 3):
         for sg in SIGS + ["SIG_RHS"]:
             L.append("    if (g.dim == %d && sig == (%s)) {" % (d, sg))
-            L.append("        if (g.uni) slot_kernel<%d, %d, %s, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);" % (d, kc, sg))
-            L.append("        else slot_kernel<%d, %d, %s, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);" % (d, kc, sg))
+            L.append("        if (g.uni) launch_pass(slot_kernel<%d, %d, %s, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);" % (d, kc, sg))
+            L.append("        else launch_pass(slot_kernel<%d, %d, %s, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);" % (d, kc, sg))
             L.append("        return (int)cudaGetLastError();")
             L.append("    }")
     L.append("    *done = false;")
@@ -251,8 +256,8 @@ def vunit(kc, fname):
     for d in (2, 3):
         for sg in FAST_SIGS:
             L.append("    if (g.dim == %d && sig == (%s)) {" % (d, sg))
-            L.append("        vec_kernel<%d, %d, %s><<<grid, VBLOCK, vec_smem<%s>(), st>>>(g, P, A, B, L, ptype);" % (d, kc, sg, sg))
-            L.append("        if (vec_crowds(g)) wide_fix_kernel<%d, %d><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);" % (d, kc))
+            L.append("        launch_pass(vec_kernel<%d, %d, %s>, grid, VBLOCK, vec_smem<%s>(), st, g, P, A, B, L, ptype);" % (d, kc, sg, sg))
+            L.append("        if (vec_crowds(g)) launch_pass(wide_fix_kernel<%d, %d>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);" % (d, kc))
             L.append("        return (int)cudaGetLastError();")
             L.append("    }")
             prep.append("    if (cudaFuncSetAttribute(vec_kernel<%d, %d, %s>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vec_smem<%s>()) != cudaSuccess) return -1;" % (d, kc, sg, sg))
@@ -285,8 +290,8 @@ def vunit(kc, fname):
     for d in (2, 3):
         for sg in FAST_SIGS:
             L.append("    if (dim == %d && sig == (%s)) {" % (d, sg))
-            L.append("        packed_kernel<%d, %d, %s><<<blocks, VBLOCK, vec_smem<%s>(), st>>>(tab, bstart, n);" % (d, kc, sg, sg))
-            L.append("        if (crowds) packed_wide_fix_kernel<%d, %d><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);" % (d, kc))
+            L.append("        launch_pass(packed_kernel<%d, %d, %s>, blocks, VBLOCK, vec_smem<%s>(), st, tab, bstart, n);" % (d, kc, sg, sg))
+            L.append("        if (crowds) launch_pass(packed_wide_fix_kernel<%d, %d>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);" % (d, kc))
             L.append("        return (int)cudaGetLastError();")
             L.append("    }")
             prep.append("    if (cudaFuncSetAttribute(packed_kernel<%d, %d, %s>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)vec_smem<%s>()) != cudaSuccess) return -1;" % (d, kc, sg, sg))

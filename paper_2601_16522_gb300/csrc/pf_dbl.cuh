@@ -683,6 +683,7 @@ __global__ void __launch_bounds__(DBL_TX *ROWS, ROWS == 8 ? 3 : 8)
 dbl_kernel(const __grid_constant__ Geom g, const __grid_constant__ Pass<double> P, const double *__restrict__ tabA,
            const double *__restrict__ tabB, const double *__restrict__ tabL, const signed char *__restrict__ ptype)
 {
+    pass_begin();
     dbl_body<DIM, KC, ROWS>(g, P, tabA, tabB, tabL, ptype);
 }
 

@@ -206,6 +206,15 @@ enum { MODE_RHS = 0, MODE_STAGE = 1, MODE_ERR = 2 };
 // no pass of a step overwrites, stays intact for the engine to return.
 enum { FLAG_SIMPLEX = 1, FLAG_NZ_OVERFLOW = 2, FLAG_TIMEOUT = 4, FLAG_NONFINITE = 8 };
 
+// Start of a pass kernel: it may be launched while the pass before it drains
+// (launch_pass), so it waits for that pass's results first, then lets the next
+// pass in.
+__device__ __forceinline__ void pass_begin()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ bool pass_skipped(const int *flag) { return *(const volatile int *)flag != 0; }
 
 __device__ __forceinline__ void raise_flag(int *flag, int bits)
@@ -2142,6 +2151,7 @@ __global__ void __launch_bounds__(BLOCK, MASK ? (KC ? PF_MASK_MINB_K1 : PF_MASK_
 fast_kernel(const __grid_constant__ Geom g, const __grid_constant__ Pass<float> P, const float *__restrict__ tabA,
             const float *__restrict__ tabB, const float *__restrict__ tabL, const signed char *__restrict__ ptype)
 {
+    pass_begin();
     fast_body<DIM, KC, SIG, NMAX, MASK>(g, P, tabA, tabB, tabL, ptype);
 }
 

@@ -843,7 +843,7 @@ __device__ __forceinline__ bool slot_fast(const Geom &g, const Pass<float> &P, S
 }
 
 // Resident blocks per SM (register budget), 256^3 x 2000 grains: 44.5 ms at 3,
-// 42.4 at 4 and 50 at 5, where 48 registers spill.
+// 42.4 at 4 and 50 at 5, where 48 registers spill; with a concentration 4 spill.
 __host__ __device__ constexpr int slot_minb(int K) { return K ? 3 : 4; }
 
 // One slot pass: one cell per thread, 32 x 8 tiles, one z plane per block.
@@ -852,6 +852,7 @@ __global__ void __launch_bounds__(BLOCK, slot_minb(KC))
 slot_kernel(const __grid_constant__ Geom g, const __grid_constant__ Pass<float> P, const float *__restrict__ tabA,
             const float *__restrict__ tabB, const float *__restrict__ tabL, const signed char *__restrict__ ptype)
 {
+    pass_begin();
     __shared__ SlotSmem<UNI, SIG> S;
     if (pass_skipped(P.flag)) return;
     const int tid = threadIdx.x;

@@ -12,35 +12,35 @@ int launch_f32k1(const Geom &g, const Pass<float> &P, unsigned sig, cudaStream_t
     const size_t smt = 1024 + sizeof(TmaSmem) + sizeof(ListSmem<float>);
     if (g.N > 32 && g.N <= 128 && g.Vs < 0x7fffffffLL) {
         if (g.dim == 2 && sig == (SIG_O2 | SIG_PROJECT)) {
-            fast_kernel<2, 1, SIG_O2 | SIG_PROJECT, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+            launch_pass(fast_kernel<2, 1, SIG_O2 | SIG_PROJECT, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 2 && sig == (SIG_Z | SIG_PROJECT)) {
-            fast_kernel<2, 1, SIG_Z | SIG_PROJECT, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+            launch_pass(fast_kernel<2, 1, SIG_Z | SIG_PROJECT, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 2 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-            fast_kernel<2, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+            launch_pass(fast_kernel<2, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 2 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-            fast_kernel<2, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+            launch_pass(fast_kernel<2, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 3 && sig == (SIG_O2 | SIG_PROJECT)) {
-            fast_kernel<3, 1, SIG_O2 | SIG_PROJECT, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+            launch_pass(fast_kernel<3, 1, SIG_O2 | SIG_PROJECT, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 3 && sig == (SIG_Z | SIG_PROJECT)) {
-            fast_kernel<3, 1, SIG_Z | SIG_PROJECT, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+            launch_pass(fast_kernel<3, 1, SIG_Z | SIG_PROJECT, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 3 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-            fast_kernel<3, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+            launch_pass(fast_kernel<3, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 3 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-            fast_kernel<3, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 128><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+            launch_pass(fast_kernel<3, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 128>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
     }
@@ -123,181 +123,181 @@ int launch_f32k1(const Geom &g, const Pass<float> &P, unsigned sig, cudaStream_t
         }
         if (g.N <= 4) {
             if (g.dim == 2 && sig == (SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_P2 | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_P2 | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_R0OUT | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_R0OUT | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_ERR)) {
-                fast_kernel<2, 1, SIG_ERR, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_ERR, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_P0 | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_P0 | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_ERR | SIG_R0OUT)) {
-                fast_kernel<2, 1, SIG_ERR | SIG_R0OUT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_ERR | SIG_R0OUT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_O2 | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_O2 | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_Z | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_Z | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_P2 | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_P2 | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_R0OUT | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_R0OUT | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_ERR)) {
-                fast_kernel<3, 1, SIG_ERR, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_ERR, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_P0 | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_P0 | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_ERR | SIG_R0OUT)) {
-                fast_kernel<3, 1, SIG_ERR | SIG_R0OUT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_ERR | SIG_R0OUT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_O2 | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_O2 | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_Z | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_Z | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 4><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 4>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
         }
         if (g.N > 4) {
             if (g.dim == 2 && sig == (SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_P2 | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_P2 | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_R0OUT | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_R0OUT | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_ERR)) {
-                fast_kernel<2, 1, SIG_ERR, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_ERR, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_P0 | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_P0 | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_ERR | SIG_R0OUT)) {
-                fast_kernel<2, 1, SIG_ERR | SIG_R0OUT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_ERR | SIG_R0OUT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_O2 | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_O2 | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_Z | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_Z | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<2, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_P2 | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_P2 | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_R0OUT | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_R0OUT | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_ERR)) {
-                fast_kernel<3, 1, SIG_ERR, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_ERR, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_P0 | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_P0 | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_ERR | SIG_R0OUT)) {
-                fast_kernel<3, 1, SIG_ERR | SIG_R0OUT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_ERR | SIG_R0OUT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_O2 | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_O2 | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_Z | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_Z | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_Z | SIG_O2 | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<3, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 32><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 1, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 32>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
         }

@@ -12,35 +12,35 @@ int launch_f64(const Geom &g, const Pass<double> &P, unsigned sig, cudaStream_t 
         const int rows = dbl_rows(g);
         const dim3 dgrid((g.nx + DBL_TX - 1) / DBL_TX, (g.ny + rows - 1) / rows, g.nz);
         if (g.dim == 2 && g.K == 0 && rows == 2) {
-            dbl_kernel<2, 0, 2><<<dgrid, DBL_TX * 2, sizeof(DblSmem<2>), st>>>(g, P, A, B, L, ptype);
+            launch_pass(dbl_kernel<2, 0, 2>, dgrid, DBL_TX * 2, sizeof(DblSmem<2>), st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 2 && g.K == 0 && rows == 8) {
-            dbl_kernel<2, 0, 8><<<dgrid, DBL_TX * 8, sizeof(DblSmem<8>), st>>>(g, P, A, B, L, ptype);
+            launch_pass(dbl_kernel<2, 0, 8>, dgrid, DBL_TX * 8, sizeof(DblSmem<8>), st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 2 && g.K == 1 && rows == 2) {
-            dbl_kernel<2, 1, 2><<<dgrid, DBL_TX * 2, sizeof(DblSmem<2>), st>>>(g, P, A, B, L, ptype);
+            launch_pass(dbl_kernel<2, 1, 2>, dgrid, DBL_TX * 2, sizeof(DblSmem<2>), st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 2 && g.K == 1 && rows == 8) {
-            dbl_kernel<2, 1, 8><<<dgrid, DBL_TX * 8, sizeof(DblSmem<8>), st>>>(g, P, A, B, L, ptype);
+            launch_pass(dbl_kernel<2, 1, 8>, dgrid, DBL_TX * 8, sizeof(DblSmem<8>), st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 3 && g.K == 0 && rows == 2) {
-            dbl_kernel<3, 0, 2><<<dgrid, DBL_TX * 2, sizeof(DblSmem<2>), st>>>(g, P, A, B, L, ptype);
+            launch_pass(dbl_kernel<3, 0, 2>, dgrid, DBL_TX * 2, sizeof(DblSmem<2>), st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 3 && g.K == 0 && rows == 8) {
-            dbl_kernel<3, 0, 8><<<dgrid, DBL_TX * 8, sizeof(DblSmem<8>), st>>>(g, P, A, B, L, ptype);
+            launch_pass(dbl_kernel<3, 0, 8>, dgrid, DBL_TX * 8, sizeof(DblSmem<8>), st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 3 && g.K == 1 && rows == 2) {
-            dbl_kernel<3, 1, 2><<<dgrid, DBL_TX * 2, sizeof(DblSmem<2>), st>>>(g, P, A, B, L, ptype);
+            launch_pass(dbl_kernel<3, 1, 2>, dgrid, DBL_TX * 2, sizeof(DblSmem<2>), st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
         if (g.dim == 3 && g.K == 1 && rows == 8) {
-            dbl_kernel<3, 1, 8><<<dgrid, DBL_TX * 8, sizeof(DblSmem<8>), st>>>(g, P, A, B, L, ptype);
+            launch_pass(dbl_kernel<3, 1, 8>, dgrid, DBL_TX * 8, sizeof(DblSmem<8>), st, g, P, A, B, L, ptype);
             return (int)cudaGetLastError();
         }
     }

@@ -12,247 +12,247 @@ int launch_m32k0(const Geom &g, const Pass<float> &P, unsigned sig, cudaStream_t
     if (g.N <= 128 && g.Vs < 0x7fffffffLL) {
         if (g.N <= 4) {
             if (g.dim == 2 && sig == (SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P2 | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P2 | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_R0OUT | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_R0OUT | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_ERR)) {
-                fast_kernel<2, 0, SIG_ERR, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_ERR, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_O2 | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_O2 | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_Z | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_Z | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P2 | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P2 | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_R0OUT | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_R0OUT | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_ERR)) {
-                fast_kernel<3, 0, SIG_ERR, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_ERR, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_O2 | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_O2 | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_Z | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_Z | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 4, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 4, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
         }
         if (g.N > 4 && g.N <= 32) {
             if (g.dim == 2 && sig == (SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P2 | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P2 | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_R0OUT | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_R0OUT | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_ERR)) {
-                fast_kernel<2, 0, SIG_ERR, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_ERR, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_O2 | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_O2 | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_Z | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_Z | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P2 | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P2 | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_R0OUT | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_R0OUT | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_ERR)) {
-                fast_kernel<3, 0, SIG_ERR, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_ERR, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_O2 | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_O2 | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_Z | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_Z | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 32, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 32, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
         }
         if (g.N > 32) {
             if (g.dim == 2 && sig == (SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P2 | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P2 | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_R0OUT | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_R0OUT | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_ERR)) {
-                fast_kernel<2, 0, SIG_ERR, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_ERR, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_O2 | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_O2 | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_Z | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_Z | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 2 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<2, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<2, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P2 | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P2 | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_R0OUT | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_R0OUT | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_ERR)) {
-                fast_kernel<3, 0, SIG_ERR, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_ERR, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_O2 | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_O2 | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_Z | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_Z | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_Z | SIG_O2 | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_Z | SIG_O2 | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
             if (g.dim == 3 && sig == (SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT)) {
-                fast_kernel<3, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 128, true><<<grid, BLOCK, smf, st>>>(g, P, A, B, L, ptype);
+                launch_pass(fast_kernel<3, 0, SIG_P0 | SIG_Z | SIG_EMB | SIG_PROJECT, 128, true>, grid, BLOCK, smf, st, g, P, A, B, L, ptype);
                 return (int)cudaGetLastError();
             }
         }

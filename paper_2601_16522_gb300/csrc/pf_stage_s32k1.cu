@@ -9,73 +9,73 @@ int launch_s32k1(const Geom &g, const Pass<float> &P, unsigned sig, cudaStream_t
     const dim3 grid(g.tiles_x, g.tiles_y, g.nz);
     *done = true;
     if (g.dim == 2 && sig == (SIG_PROJECT)) {
-        if (g.uni) slot_kernel<2, 1, SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<2, 1, SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<2, 1, SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<2, 1, SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_P2 | SIG_PROJECT)) {
-        if (g.uni) slot_kernel<2, 1, SIG_P2 | SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<2, 1, SIG_P2 | SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<2, 1, SIG_P2 | SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<2, 1, SIG_P2 | SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-        if (g.uni) slot_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-        if (g.uni) slot_kernel<2, 1, SIG_R0OUT | SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<2, 1, SIG_R0OUT | SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<2, 1, SIG_R0OUT | SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<2, 1, SIG_R0OUT | SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_ERR)) {
-        if (g.uni) slot_kernel<2, 1, SIG_ERR, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<2, 1, SIG_ERR, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<2, 1, SIG_ERR, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<2, 1, SIG_ERR, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_P0 | SIG_PROJECT)) {
-        if (g.uni) slot_kernel<2, 1, SIG_P0 | SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<2, 1, SIG_P0 | SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<2, 1, SIG_P0 | SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<2, 1, SIG_P0 | SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_RHS)) {
-        if (g.uni) slot_kernel<2, 1, SIG_RHS, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<2, 1, SIG_RHS, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<2, 1, SIG_RHS, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<2, 1, SIG_RHS, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_PROJECT)) {
-        if (g.uni) slot_kernel<3, 1, SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<3, 1, SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<3, 1, SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<3, 1, SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_P2 | SIG_PROJECT)) {
-        if (g.uni) slot_kernel<3, 1, SIG_P2 | SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<3, 1, SIG_P2 | SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<3, 1, SIG_P2 | SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<3, 1, SIG_P2 | SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-        if (g.uni) slot_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-        if (g.uni) slot_kernel<3, 1, SIG_R0OUT | SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<3, 1, SIG_R0OUT | SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<3, 1, SIG_R0OUT | SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<3, 1, SIG_R0OUT | SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_ERR)) {
-        if (g.uni) slot_kernel<3, 1, SIG_ERR, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<3, 1, SIG_ERR, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<3, 1, SIG_ERR, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<3, 1, SIG_ERR, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_P0 | SIG_PROJECT)) {
-        if (g.uni) slot_kernel<3, 1, SIG_P0 | SIG_PROJECT, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<3, 1, SIG_P0 | SIG_PROJECT, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<3, 1, SIG_P0 | SIG_PROJECT, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<3, 1, SIG_P0 | SIG_PROJECT, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_RHS)) {
-        if (g.uni) slot_kernel<3, 1, SIG_RHS, true><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
-        else slot_kernel<3, 1, SIG_RHS, false><<<grid, BLOCK, 0, st>>>(g, P, A, B, L, ptype);
+        if (g.uni) launch_pass(slot_kernel<3, 1, SIG_RHS, true>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
+        else launch_pass(slot_kernel<3, 1, SIG_RHS, false>, grid, BLOCK, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     *done = false;

@@ -9,73 +9,73 @@ int launch_v32k1(const Geom &g, const Pass<float> &P, unsigned sig, cudaStream_t
     const dim3 grid((g.nx + 2 * VTX - 1) / (2 * VTX), (g.ny + VTY - 1) / VTY, g.nz);
     *done = true;
     if (g.dim == 2 && sig == (SIG_PROJECT)) {
-        vec_kernel<2, 1, SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<2, 1, SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_P2 | SIG_PROJECT)) {
-        vec_kernel<2, 1, SIG_P2 | SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_P2 | SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<2, 1, SIG_P2 | SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_P2 | SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-        vec_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-        vec_kernel<2, 1, SIG_R0OUT | SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_R0OUT | SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<2, 1, SIG_R0OUT | SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_R0OUT | SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_ERR)) {
-        vec_kernel<2, 1, SIG_ERR><<<grid, VBLOCK, vec_smem<SIG_ERR>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<2, 1, SIG_ERR>, grid, VBLOCK, vec_smem<SIG_ERR>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_P0 | SIG_PROJECT)) {
-        vec_kernel<2, 1, SIG_P0 | SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_P0 | SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<2, 1, SIG_P0 | SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_P0 | SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 2 && sig == (SIG_ERR | SIG_R0OUT)) {
-        vec_kernel<2, 1, SIG_ERR | SIG_R0OUT><<<grid, VBLOCK, vec_smem<SIG_ERR | SIG_R0OUT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<2, 1, SIG_ERR | SIG_R0OUT>, grid, VBLOCK, vec_smem<SIG_ERR | SIG_R0OUT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_PROJECT)) {
-        vec_kernel<3, 1, SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<3, 1, SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_P2 | SIG_PROJECT)) {
-        vec_kernel<3, 1, SIG_P2 | SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_P2 | SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<3, 1, SIG_P2 | SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_P2 | SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-        vec_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-        vec_kernel<3, 1, SIG_R0OUT | SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_R0OUT | SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<3, 1, SIG_R0OUT | SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_R0OUT | SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_ERR)) {
-        vec_kernel<3, 1, SIG_ERR><<<grid, VBLOCK, vec_smem<SIG_ERR>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<3, 1, SIG_ERR>, grid, VBLOCK, vec_smem<SIG_ERR>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_P0 | SIG_PROJECT)) {
-        vec_kernel<3, 1, SIG_P0 | SIG_PROJECT><<<grid, VBLOCK, vec_smem<SIG_P0 | SIG_PROJECT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<3, 1, SIG_P0 | SIG_PROJECT>, grid, VBLOCK, vec_smem<SIG_P0 | SIG_PROJECT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     if (g.dim == 3 && sig == (SIG_ERR | SIG_R0OUT)) {
-        vec_kernel<3, 1, SIG_ERR | SIG_R0OUT><<<grid, VBLOCK, vec_smem<SIG_ERR | SIG_R0OUT>(), st>>>(g, P, A, B, L, ptype);
-        if (vec_crowds(g)) wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(g, P, A, B, L, ptype);
+        launch_pass(vec_kernel<3, 1, SIG_ERR | SIG_R0OUT>, grid, VBLOCK, vec_smem<SIG_ERR | SIG_R0OUT>(), st, g, P, A, B, L, ptype);
+        if (vec_crowds(g)) launch_pass(wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, g, P, A, B, L, ptype);
         return (int)cudaGetLastError();
     }
     *done = false;
@@ -136,73 +136,73 @@ int launchp_v32k1(int dim, unsigned sig, const VecInst *tab, const int *bstart, 
 {
     *ok = true;
     if (dim == 2 && sig == (SIG_PROJECT)) {
-        packed_kernel<2, 1, SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<2, 1, SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 2 && sig == (SIG_P2 | SIG_PROJECT)) {
-        packed_kernel<2, 1, SIG_P2 | SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_P2 | SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<2, 1, SIG_P2 | SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_P2 | SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 2 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-        packed_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<2, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 2 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-        packed_kernel<2, 1, SIG_R0OUT | SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_R0OUT | SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<2, 1, SIG_R0OUT | SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_R0OUT | SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 2 && sig == (SIG_ERR)) {
-        packed_kernel<2, 1, SIG_ERR><<<blocks, VBLOCK, vec_smem<SIG_ERR>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<2, 1, SIG_ERR>, blocks, VBLOCK, vec_smem<SIG_ERR>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 2 && sig == (SIG_P0 | SIG_PROJECT)) {
-        packed_kernel<2, 1, SIG_P0 | SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_P0 | SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<2, 1, SIG_P0 | SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_P0 | SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 2 && sig == (SIG_ERR | SIG_R0OUT)) {
-        packed_kernel<2, 1, SIG_ERR | SIG_R0OUT><<<blocks, VBLOCK, vec_smem<SIG_ERR | SIG_R0OUT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<2, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<2, 1, SIG_ERR | SIG_R0OUT>, blocks, VBLOCK, vec_smem<SIG_ERR | SIG_R0OUT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<2, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 3 && sig == (SIG_PROJECT)) {
-        packed_kernel<3, 1, SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<3, 1, SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 3 && sig == (SIG_P2 | SIG_PROJECT)) {
-        packed_kernel<3, 1, SIG_P2 | SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_P2 | SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<3, 1, SIG_P2 | SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_P2 | SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 3 && sig == (SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT)) {
-        packed_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<3, 1, SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_P0 | SIG_P2 | SIG_R0IN | SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 3 && sig == (SIG_R0OUT | SIG_PROJECT)) {
-        packed_kernel<3, 1, SIG_R0OUT | SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_R0OUT | SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<3, 1, SIG_R0OUT | SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_R0OUT | SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 3 && sig == (SIG_ERR)) {
-        packed_kernel<3, 1, SIG_ERR><<<blocks, VBLOCK, vec_smem<SIG_ERR>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<3, 1, SIG_ERR>, blocks, VBLOCK, vec_smem<SIG_ERR>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 3 && sig == (SIG_P0 | SIG_PROJECT)) {
-        packed_kernel<3, 1, SIG_P0 | SIG_PROJECT><<<blocks, VBLOCK, vec_smem<SIG_P0 | SIG_PROJECT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<3, 1, SIG_P0 | SIG_PROJECT>, blocks, VBLOCK, vec_smem<SIG_P0 | SIG_PROJECT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     if (dim == 3 && sig == (SIG_ERR | SIG_R0OUT)) {
-        packed_kernel<3, 1, SIG_ERR | SIG_R0OUT><<<blocks, VBLOCK, vec_smem<SIG_ERR | SIG_R0OUT>(), st>>>(tab, bstart, n);
-        if (crowds) packed_wide_fix_kernel<3, 1><<<WIDE_FIX_BLOCKS, VCELLS, 0, st>>>(tab, n, done);
+        launch_pass(packed_kernel<3, 1, SIG_ERR | SIG_R0OUT>, blocks, VBLOCK, vec_smem<SIG_ERR | SIG_R0OUT>(), st, tab, bstart, n);
+        if (crowds) launch_pass(packed_wide_fix_kernel<3, 1>, WIDE_FIX_BLOCKS, VCELLS, 0, st, tab, n, done);
         return (int)cudaGetLastError();
     }
     *ok = false;

@@ -898,6 +898,7 @@ __global__ void __launch_bounds__(VCELLS)
 wide_fix_kernel(const __grid_constant__ Geom g, const __grid_constant__ Pass<float> P, const float *__restrict__ tabA,
                 const float *__restrict__ tabB, const float *__restrict__ tabL, const signed char *__restrict__ ptype)
 {
+    pass_begin();
     wide_fix_body<DIM, KC>(g, P, tabA, tabB, tabL, ptype);
 }
 
@@ -926,6 +927,7 @@ __global__ void __launch_bounds__(VBLOCK, (vec_minb<KC, SIG>()))
 vec_kernel(const __grid_constant__ Geom g, const __grid_constant__ Pass<float> P, const float *__restrict__ tabA,
            const float *__restrict__ tabB, const float *__restrict__ tabL, const signed char *__restrict__ ptype)
 {
+    pass_begin();
     vec_body<DIM, KC, SIG>(g, P, tabA, tabB, tabL, ptype, blockIdx.x, blockIdx.y, blockIdx.z,
                            (int)(gridDim.x * gridDim.y * gridDim.z));
 }
@@ -975,6 +977,7 @@ template <int DIM, int KC, unsigned SIG>
 __global__ void __launch_bounds__(VBLOCK, (vec_minb<KC, SIG>()))
 packed_kernel(const VecInst *__restrict__ tab, const int *__restrict__ bstart, int n)
 {
+    pass_begin();
     __shared__ Geom gs;
     __shared__ Pass<float> Ps;
     // the block's problem: the last k with bstart[k] <= block (prefix sums
@@ -1003,6 +1006,7 @@ template <int DIM, int KC>
 __global__ void __launch_bounds__(VCELLS)
 packed_wide_fix_kernel(const VecInst *__restrict__ tab, int n, int *done)
 {
+    pass_begin();
     for (int k = 0; k < n; ++k) {
         const VecInst &I = tab[k];
         if (!vec_crowds(I.g)) continue;
