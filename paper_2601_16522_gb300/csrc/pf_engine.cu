@@ -43,13 +43,13 @@ template <typename T>
 __global__ void pack_kernel(const double *__restrict__ phi, const double *__restrict__ c, T *__restrict__ dst,
                             long long V, long long Vs, int N, int NF, double cref)
 {
-    const long long n = V * NF;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-         k += (long long)gridDim.x * blockDim.x) {
-        const long long f = k / V;
-        const long long i = k - f * V;
-        dst[f * Vs + i] = (T)(f < N ? phi[k] : c[i] - cref);
-    }
+    const int f = blockIdx.y;
+    const double *__restrict__ src = f < N ? phi + (long long)f * V : c;
+    const double ref = f < N ? 0.0 : cref;
+    T *__restrict__ out = dst + (long long)f * Vs;
+#pragma unroll 4
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x)
+        out[i] = (T)(f < N ? src[i] : src[i] - ref);
 }
 
 // pack_kernel for state vectors with segment words (pf_vec.cuh): one warp per
@@ -118,15 +118,23 @@ template <typename T>
 __global__ void unpack_kernel(const T *__restrict__ src, double *__restrict__ phi, double *__restrict__ c, long long V,
                               long long Vs, int N, int NF, double cref)
 {
-    const long long n = V * NF;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-         k += (long long)gridDim.x * blockDim.x) {
-        const long long f = k / V;
-        const long long i = k - f * V;
-        const double v = (double)src[f * Vs + i];
-        if (f < N) phi[k] = v;
-        else if (c) c[i] = v + cref;
+    const int f = blockIdx.y;
+    const T *__restrict__ in = src + (long long)f * Vs;
+    double *__restrict__ out = f < N ? phi + (long long)f * V : c;
+    if (!out) return;
+#pragma unroll 4
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x) {
+        const double v = (double)in[i];
+        out[i] = f < N ? v : v + cref;
     }
+}
+
+// Grid of the two conversions above: a row of blocks per field (one row over
+// all fields cost a 64-bit division per entry, as long as its memory time).
+dim3 field_grid(long long V, int NF)
+{
+    const long long b = (V + 255) / 256, most = 16384 / NF > 16 ? 16384 / NF : 16;
+    return dim3((unsigned)(b < most ? b : most), NF);
 }
 
 // Slot storage (pf_slots.cuh layout).  Dense ABI layout -> slots: a cell's
@@ -281,17 +289,28 @@ __global__ void finalize_err_kernel(const double *__restrict__ ps, const long lo
     if (threadIdx.x == 0) { *out_sum = ss[0]; *out_cnt = sc[0]; }
 }
 
-// Occupancy words of an FP32 state (masked storage): bit b of word w of cell
-// i (plane w) is set where phase 32 w + b is nonzero.
-__global__ void mask_kernel(const float *__restrict__ u, unsigned *__restrict__ m, long long V, long long Vs, int N)
+// pack_kernel for masked storage: the values of a cell and its occupancy words
+// (bit b of word w, plane w of m, set where phase 32 w + b is nonzero) in one
+// pass over the state; words taken from the packed planes afterwards read every
+// plane again (192^3 x 32 grains, state in and out: 0.7 of 9.9 ms with the
+// conversions by field_grid).
+__global__ void __launch_bounds__(256)
+pack_mask_kernel(const double *__restrict__ phi, const double *__restrict__ c, float *__restrict__ dst,
+                 unsigned *__restrict__ m, long long V, long long Vs, int N, int K, double cref)
 {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < V; i += (long long)gridDim.x * blockDim.x) {
         for (int w = 0; 32 * w < N; ++w) {
+            const int n = N - 32 * w < 32 ? N - 32 * w : 32;
             unsigned bits = 0u;
-            for (int b = 0; b < 32 && 32 * w + b < N; ++b)
-                if (u[(long long)(32 * w + b) * Vs + i] != 0.0f) bits |= 1u << b;
+#pragma unroll 8
+            for (int b = 0; b < n; ++b) {
+                const float v = (float)phi[(long long)(32 * w + b) * V + i];
+                dst[(long long)(32 * w + b) * Vs + i] = v;
+                if (v != 0.0f) bits |= 1u << b;
+            }
             m[(long long)w * Vs + i] = bits;
         }
+        if (K) dst[(long long)N * Vs + i] = (float)(c[i] - cref);
     }
 }
 
@@ -303,12 +322,21 @@ __global__ void totals_kernel(const T *__restrict__ u, long long V, long long Vs
     const long long chunk = (V + gridDim.x - 1) / gridDim.x;
     const long long lo = blockIdx.x * chunk;
     const long long hi = lo + chunk < V ? lo + chunk : V;
+    // +0 adds nothing and is a candidate for the maximum once: it stays off the
+    // FP64 pipe (two lanes a clock and SM), which the 30 of 32 phases absent from
+    // a cell kept busy (monitoring 128^3 x 32: 2.45 -> 1.82 ms with the energy and
+    // N_z over the phases near a cell).
     double s = 0.0, m = -1e300;
+    bool zero = false;
+#pragma unroll 4
     for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        const double v = (double)u[(long long)f * Vs + i];
+        const T t = u[(long long)f * Vs + i];
+        if (pfk::zbits(t)) { zero = true; continue; }
+        const double v = (double)t;
         s += v;
         m = v > m ? v : m;
     }
+    if (zero && 0.0 > m) m = 0.0;
     __shared__ double ss[256], sm[256];
     ss[threadIdx.x] = s;
     sm[threadIdx.x] = m;
@@ -454,6 +482,69 @@ constexpr int EMAX = 32;
 __device__ __forceinline__ bool nonzero_value(float x) { return x != 0.0f; }
 __device__ __forceinline__ bool nonzero_value(double x) { return (__double_as_longlong(x) << 1) != 0; }
 
+// Word w of the phases that can be nonzero at cell (x, y, z) or at one of its
+// face neighbours: from the segment words (pf_vec.cuh) where the state has
+// them, every phase otherwise.
+template <typename T>
+__device__ __forceinline__ unsigned near_phases(const Geom &g, const T *u, int x, int y, int z, int w)
+{
+    const unsigned full = pfk::word_bits(g.N, w);
+    if (!g.seg) return full;
+    const int sh = g.segc == 64 ? 6 : 5, tx = (g.nx + g.segc - 1) >> sh;
+    auto word = [&](int xx, int yy, int zz) {
+        return __ldg(pfk::seg_at(g, u, (zz * g.ny + yy) * tx + (xx >> sh), pfk::SEG_ANY) + w);
+    };
+    // (a neighbour across any boundary is looked up around the corner: at worst
+    // a phase too many)
+    const int xl = x > 0 ? x - 1 : g.nx - 1, xr = x < g.nx - 1 ? x + 1 : 0;
+    unsigned m = word(x, y, z);
+    if ((xl >> sh) != (x >> sh)) m |= word(xl, y, z);
+    if ((xr >> sh) != (x >> sh)) m |= word(xr, y, z);
+    m |= word(x, y > 0 ? y - 1 : g.ny - 1, z) | word(x, y < g.ny - 1 ? y + 1 : 0, z);
+    if (g.dim == 3) m |= word(x, y, z > 0 ? z - 1 : g.nz - 1) | word(x, y, z < g.nz - 1 ? z + 1 : 0);
+    return m & full;
+}
+
+// a / b with rb = 1 / b, the same bits (div_by) wherever nothing can under- or
+// overflow on the way.
+__device__ __forceinline__ double div_near(double a, double b, double rb)
+{
+    const int ex = (__double2hiint(a) >> 20) & 0x7ff;
+    return ex > 200 && ex < 1800 ? pfk::div_by(a, b, rb) : a / b;
+}
+
+// N_z of every cell of an FP32 state with segment words: the count of the
+// activity filter alone, over the phases near the cell, instead of a whole RHS
+// evaluation over all of them.
+template <int DIM>
+__global__ void __launch_bounds__(256)
+count_phases_kernel(const Geom g, const float *__restrict__ u, unsigned char *__restrict__ nz_out, int *flag)
+{
+    constexpr int NFACE = 2 * DIM;
+    if (pfk::pass_skipped(flag)) return;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.V; i += stride) {
+        const int x = (int)(i % g.nx);
+        const int y = (int)((i / g.nx) % g.ny);
+        const int z = (int)(i / ((long long)g.nx * g.ny));
+        long long off[6];
+        int ghost[6];
+        pfk::face_offsets(g, x, y, z, off, ghost);
+        int n = 0;
+        for (int w = 0; w < pfk::seg_words(g.N); ++w)
+            for (unsigned m = near_phases(g, u, x, y, z, w); m; m &= m - 1u) {
+                const float *f = u + (long long)(32 * w + __ffs(m) - 1) * g.Vs + i;
+                const float v = __ldg(f);
+                float nb[NFACE];
+#pragma unroll
+                for (int k = 0; k < NFACE; ++k) nb[k] = ghost[k] ? v : __ldg(f + off[k]);
+                if (pfk::nontrivial<NFACE>(v, nb)) ++n;
+            }
+        if (n > pfk::WIDEACT) pfk::raise_flag(flag, pfk::FLAG_NZ_OVERFLOW);
+        nz_out[i] = (unsigned char)n;
+    }
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256)
 energy_kernel(const Geom g, const T *__restrict__ u, const double *__restrict__ A, const double *__restrict__ B,
@@ -463,6 +554,7 @@ energy_kernel(const Geom g, const T *__restrict__ u, const double *__restrict__ 
     double ph[EMAX], gr[EMAX][3];
     double esum = 0.0;
     long long over = 0;
+    const double rdx = 1.0 / dx;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.V; i += stride) {
         const int x = (int)(i % g.nx);
@@ -473,7 +565,9 @@ energy_kernel(const Geom g, const T *__restrict__ u, const double *__restrict__ 
         pfk::face_offsets(g, x, y, z, off, ghost);
         int n = 0;
         bool full = false;
-        for (int a = 0; a < g.N; ++a) {
+        for (int w = 0; 32 * w < g.N && !full; ++w)
+        for (unsigned m = near_phases(g, u, x, y, z, w); m; m &= m - 1u) {
+            const int a = 32 * w + __ffs(m) - 1;
             const T *f = u + (long long)a * g.Vs + i;
             const T vt = f[0];
             T wt[3] = {vt, vt, vt};
@@ -487,7 +581,7 @@ energy_kernel(const Geom g, const T *__restrict__ u, const double *__restrict__ 
             const double v = (double)vt;
             double d[3] = {0.0, 0.0, 0.0};
             for (int ax = 0; ax < g.dim; ++ax)
-                if (wt[ax] != vt) d[ax] = __dsub_rn((double)wt[ax], v) / dx;
+                if (wt[ax] != vt) d[ax] = div_near(__dsub_rn((double)wt[ax], v), dx, rdx);
             if (n == EMAX) { full = true; break; }
             id[n] = (unsigned char)a;
             ph[n] = v;
@@ -1879,15 +1973,14 @@ int set_state_t(pf_handle *h, const double *phi_dev, const double *c_dev)
     if (h->g.seg)
         pack_seg_kernel<T><<<(unsigned)((pfk::seg_count(h->g) + 7) / 8), 256, 0, h->stream>>>(h->g, phi_dev, c_dev,
                                                                                             (T *)h->buf[h->iu]);
+    else if (h->masked)
+        pack_mask_kernel<<<grid_for(h->V), 256, 0, h->stream>>>(phi_dev, c_dev, (float *)h->buf[h->iu],
+                                                                mask_plane(h, h->buf[h->iu]), h->V, h->Vs, h->N, h->K,
+                                                                h->g.cref);
     else
-        pack_kernel<T><<<grid_for(h->V * h->NP), 256, 0, h->stream>>>(phi_dev, c_dev, (T *)h->buf[h->iu], h->V, h->Vs,
+        pack_kernel<T><<<field_grid(h->V, h->NP), 256, 0, h->stream>>>(phi_dev, c_dev, (T *)h->buf[h->iu], h->V, h->Vs,
                                                                         h->N, h->NP, h->g.cref);
     h->launches++;
-    if (h->masked) {
-        mask_kernel<<<grid_for(h->V), 256, 0, h->stream>>>((const float *)h->buf[h->iu], mask_plane(h, h->buf[h->iu]),
-                                                           h->V, h->Vs, h->N);
-        h->launches++;
-    }
     return cuda_status(cudaGetLastError());
 }
 
@@ -1900,7 +1993,7 @@ int get_state_t(pf_handle *h, double *phi_dev, double *c_dev)
         h->launches++;
         return cuda_status(cudaGetLastError());
     }
-    unpack_kernel<T><<<grid_for(h->V * h->NP), 256, 0, h->stream>>>((const T *)h->buf[h->iu], phi_dev, c_dev, h->V,
+    unpack_kernel<T><<<field_grid(h->V, h->NP), 256, 0, h->stream>>>((const T *)h->buf[h->iu], phi_dev, c_dev, h->V,
                                                                       h->Vs, h->N, h->NP, h->g.cref);
     h->launches++;
     return cuda_status(cudaGetLastError());
@@ -1917,6 +2010,13 @@ int rhs_t(pf_handle *h, unsigned char *nz_dev, bool rhs)
         cudaMemsetAsync(h->staging, 0, sizeof(double) * (size_t)h->NP * h->V, h->stream) != cudaSuccess)
         return PF_EDEVICE;
     h->cur_kind = PF_PASS_RHS;
+    if (sizeof(T) == 4 && h->g.seg && nz_dev && !rhs) {
+        const float *u = (const float *)h->buf[h->iu];
+        if (h->g.dim == 2) count_phases_kernel<2><<<grid_for(h->V), 256, 0, h->stream>>>(h->g, u, nz_dev, h->dflag);
+        else count_phases_kernel<3><<<grid_for(h->V), 256, 0, h->stream>>>(h->g, u, nz_dev, h->dflag);
+        h->launches++;
+        return cuda_status(cudaGetLastError());
+    }
     Pass<T> P = blank_pass<T>(h);
     P.mode = pfk::MODE_RHS;
     P.in = (const T *)h->buf[h->iu];
