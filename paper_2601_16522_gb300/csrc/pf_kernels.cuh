@@ -1396,7 +1396,9 @@ __device__ __forceinline__ void uni_rhs(int nz, const float (&t)[R], const float
             const float q = s + uL * (d[k] - d[k2]);
             s = k2 < nz ? q : s;
         }
-        rk[k] = nz > 1 ? -(s * inz) : 0.0f;
+        // (rounded here: the error sweep adds it to F^n, and a fused form would
+        // give the norm other bits than the loops over the tables)
+        rk[k] = nz > 1 ? -__fmul_rn(s, inz) : 0.0f;
     }
 }
 

@@ -29,7 +29,8 @@ namespace pfk {
 
 constexpr int VTX = 32;              // threads along x: 64 cells
 // Rows per block (4; measured at 256^3 x 32: 2 rows at 10/14 blocks per SM
-// and 8 rows at 2/3 give RKL2 passes of 2.13 and 2.43 ms against 2.11 ms).
+// and 8 rows at 2/3 gave RKL2 passes of 2.13 and 2.43 ms against 2.11 ms when
+// every phase was visited).
 #ifndef PF_VEC_TY
 #define PF_VEC_TY 4
 #endif
